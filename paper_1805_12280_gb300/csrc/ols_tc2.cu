@@ -317,9 +317,9 @@ __device__ inline double2 expi(int64_t num, int den)
 __global__ void tc2_constants_kernel(unsigned char *cst)
 {
     const int id = blockIdx.x * blockDim.x + threadIdx.x;
-    if (id < 64 * 64) {   // B1[j][k]: j = 4q + 2ro + e (output n1 = 2q + e, part ro), k = 2 k1 + ri
+    if (id < 64 * 64) {   // B1[j][k]: j = 4q + 2ro + e (output n1 = 2q + e, part ro), k likewise (k1, ri)
         const int j = id / 64, k = id % 64;
-        const int n1 = 2 * (j / 4) + (j & 1), ro = (j / 2) & 1, k1 = k / 2, ri = k & 1;
+        const int n1 = 2 * (j / 4) + (j & 1), ro = (j / 2) & 1, k1 = 2 * (k / 4) + (k & 1), ri = (k / 2) & 1;
         const double2 w = expi((int64_t)n1 * k1, 32);
         const double v = ro == 0 ? (ri == 0 ? w.x : -w.y) : (ri == 0 ? w.y : w.x);
         reinterpret_cast<__half *>(cst + CB_B1)[b1_off(j, k) / 2] = __double2half(v);
@@ -359,8 +359,10 @@ __global__ void tc2_pretransform_kernel(const float2 *__restrict__ h32, int M, i
         re = ldexp(re, eH);
         im = ldexp(im, eH);
     }
-    __half2 *dst = reinterpret_cast<__half2 *>(H16 + (size_t)z * H_BYTES + (size_t)k2 * H_ROW) + k1;
-    *dst = __halves2half2(__double2half(re), __double2half(im));
+    // pairs of k1 per 32-bit word: word 2j = (re 2j, re 2j + 1), word 2j + 1 = (im 2j, im 2j + 1)
+    __half *dst = reinterpret_cast<__half *>(H16 + (size_t)z * H_BYTES + (size_t)k2 * H_ROW) + 4 * (k1 / 2) + (k1 & 1);
+    dst[0] = __double2half(re);
+    dst[2] = __double2half(im);
 }
 
 }  // namespace tc2
@@ -470,15 +472,16 @@ __device__ __forceinline__ void tc2_body(const Src &src, const tc2::Args &a)
                 mbar_arrive(&bar[B_SCALE0 + (il & 1)]);
             }
             PSync::sync();   // spectra in natural order visible
-            __half2 x[32], xs[32];
+            __half2 xr[16], xi[16], nxi[16];   // (k1 = 2j, 2j + 1) pairs of re, im and -im
             {
                 const float f = ldexpf(1.f, sg ? ex[1] : ex[0]);
                 const float2 *Xs = segb + sg * L + k2;
 #pragma unroll
-                for (int k1 = 0; k1 < 32; ++k1) {
-                    const float2 c = Xs[64 * k1];
-                    x[k1] = __floats2half2_rn(c.x * f, c.y * f);
-                    xs[k1] = __floats2half2_rn(-c.y * f, c.x * f);
+                for (int j = 0; j < 16; ++j) {
+                    const float2 c0 = Xs[128 * j], c1 = Xs[128 * j + 64];
+                    xr[j] = __floats2half2_rn(c0.x * f, c1.x * f);
+                    xi[j] = __floats2half2_rn(c0.y * f, c1.y * f);
+                    nxi[j] = __hneg2(xi[j]);
                 }
             }
             mbar_arrive(&bar[B_SEG_FREE]);
@@ -497,13 +500,17 @@ __device__ __forceinline__ void tc2_body(const Src &src, const tc2::Args &a)
                     uint32_t y[32];
 #pragma unroll
                     for (int c = 0; c < 8; ++c) {
-                        const uint4 hv = hrow[c];
+                        const uint4 hv = hrow[c];   // re, im of the pair j = 2 c, then of 2 c + 1
                         const uint32_t hw[4] = {hv.x, hv.y, hv.z, hv.w};
 #pragma unroll
-                        for (int i = 0; i < 4; ++i) {
-                            const __half2 h = *reinterpret_cast<const __half2 *>(&hw[i]);
-                            const __half2 r = __hfma2(__low2half2(h), x[4 * c + i], __hmul2(__high2half2(h), xs[4 * c + i]));
-                            y[4 * c + i] = *reinterpret_cast<const uint32_t *>(&r);
+                        for (int i = 0; i < 2; ++i) {
+                            const int j = 2 * c + i;
+                            const __half2 hr = *reinterpret_cast<const __half2 *>(&hw[2 * i]);
+                            const __half2 hi = *reinterpret_cast<const __half2 *>(&hw[2 * i + 1]);
+                            const __half2 yr = __hfma2(hr, xr[j], __hmul2(hi, nxi[j]));
+                            const __half2 yi = __hfma2(hr, xi[j], __hmul2(hi, xr[j]));
+                            y[2 * j] = *reinterpret_cast<const uint32_t *>(&yr);
+                            y[2 * j + 1] = *reinterpret_cast<const uint32_t *>(&yi);
                         }
                     }
                     __syncwarp();
