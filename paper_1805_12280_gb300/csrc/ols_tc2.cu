@@ -666,32 +666,48 @@ __device__ __forceinline__ void tc2_body(const Src &src, const tc2::Args &a)
 #pragma unroll
                         for (int g = 1; g < 8; ++g) mx = fmaxf(mx, fmaxf(pw[g].x, pw[g].y));
                         if (!__any_sync(0xffffffffu, mx > a.threshold)) continue;   // most chunks: no crossing
+                        // A lane's crossings as a bit mask, with the value of the highest one: one pass
+                        // of compares and selects, no vote per output.  Lanes then append one record
+                        // a round (one round unless a lane holds several crossings).
                         const int c0 = 512 * cc - (a.K - 1);
-                        const bool whole = c0 >= 0 && c0 + 511 < lim;   // every output of the chunk is kept
+                        unsigned m = 0;
+                        float val = 0.f;
+                        if (c0 >= 0 && c0 + 511 < lim) {   // every output of the chunk is kept
 #pragma unroll
-                        for (int g = 0; g < 8; ++g) {
-                            const int t0 = tbase + 32 * (16 * cc + 2 * g);
-                            const bool cx = pw[g].x > a.threshold && (whole || (unsigned)t0 < (unsigned)lim);
-                            const bool cy = pw[g].y > a.threshold && (whole || (unsigned)(t0 + 32) < (unsigned)lim);
-                            const unsigned bx = __ballot_sync(0xffffffffu, cx), by = __ballot_sync(0xffffffffu, cy);
-                            if ((bx | by) == 0) continue;
-                            const unsigned nx = __popc(bx), nxy = nx + __popc(by);
-                            if (nst + nxy > (unsigned)CAND_STAGE) flush_stage();
-                            if (cx) {
+                            for (int g = 0; g < 8; ++g) {
+                                if (pw[g].x > a.threshold) { m |= 1u << (2 * g); val = pw[g].x; }
+                                if (pw[g].y > a.threshold) { m |= 2u << (2 * g); val = pw[g].y; }
+                            }
+                        } else {
+#pragma unroll
+                            for (int g = 0; g < 8; ++g) {
+                                const int t0 = tbase + 32 * (16 * cc + 2 * g);
+                                if (pw[g].x > a.threshold && (unsigned)t0 < (unsigned)lim) { m |= 1u << (2 * g); val = pw[g].x; }
+                                if (pw[g].y > a.threshold && (unsigned)(t0 + 32) < (unsigned)lim) { m |= 2u << (2 * g); val = pw[g].y; }
+                            }
+                        }
+                        unsigned act = __ballot_sync(0xffffffffu, m != 0);
+                        while (act) {
+                            const unsigned na = __popc(act);
+                            if (nst + na > (unsigned)CAND_STAGE) flush_stage();
+                            if (m) {
+                                const int j = 31 - __clz(m);
                                 fdas_candidate c;
                                 c.tpl = z;
-                                c.power = pw[g].x;
-                                c.bin = segrow + t0;
-                                stg[nst + __popc(bx & lt)] = c;
+                                c.power = val;
+                                c.bin = segrow + tbase + 32 * (16 * cc + j);
+                                stg[nst + __popc(act & lt)] = c;
+                                m ^= 1u << j;
                             }
-                            if (cy) {
-                                fdas_candidate c;
-                                c.tpl = z;
-                                c.power = pw[g].y;
-                                c.bin = segrow + t0 + 32;
-                                stg[nst + nx + __popc(by & lt)] = c;
+                            nst += na;
+                            act = __ballot_sync(0xffffffffu, m != 0);
+                            if (act) {   // some lane has more: the value of its next crossing
+#pragma unroll
+                                for (int g = 0; g < 8; ++g) {
+                                    if (m & (1u << (2 * g))) val = pw[g].x;
+                                    if (m & (2u << (2 * g))) val = pw[g].y;
+                                }
                             }
-                            nst += nxy;
                         }
                         continue;
                     }
