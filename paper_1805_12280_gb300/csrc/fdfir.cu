@@ -29,6 +29,10 @@ constexpr size_t col_smem_bytes()
 {
     return sizeof(float2) * ((size_t)P1 * TBP + P1 + 16 * (NT1 + 1));
 }
+constexpr int CT_INV = 4;   // columns per block of the inverse column pass
+constexpr size_t col_inv_smem_bytes() { return sizeof(float2) * (16 * (NT1 + 1) + 8) * CT_INV; }
+template <int P2>
+constexpr size_t row_inv_smem_bytes() { return sizeof(float2) * 16 * (P2 / 16 + 1); }
 template <int P2>
 constexpr size_t row_smem_bytes()
 {
@@ -103,54 +107,106 @@ __global__ void __launch_bounds__(P2 / 16) fdfir_row_fwd(float2 *__restrict__ A,
     for (int j = 0; j < 16; ++j) row[j * NT2 + tid] = X[j];
 }
 
+// Inverse L-point FFT (unnormalised) of CT independent transforms by L/16 threads each, thread
+// (t, column) from the C distribution the forward transform leaves to natural order, v[a] =
+// y[a NT + t].  Passes C', B', A' with the twiddles of B' and A' folded into the butterflies
+// (dft_twiddled: 16 factors read per thread instead of 31 twiddles); both exchanges go through
+// `ex` (16 (NT + 1) CT values, the columns side by side), free on entry, with a barrier between
+// the reads of the first and the stores of the second: half the shared memory, so that twice as
+// many blocks share an SM.
+template <int L, int CT>
+__device__ __forceinline__ void inverse_fft_folded(float2 (&v)[16], float2 *ex, const float2 *__restrict__ tw, int t, int col)
+{
+    using Gm = Geo<L>;
+    constexpr int NT = Gm::NT, Q = Gm::Q, R = Gm::R, GB = Gm::GB, GC = Gm::GC, LD = NT + 1, MASK = L - 1;
+    const int k1 = t & 15, hi = t >> 4;
+    dft<R, 1, 1, 0>(v);
+    if constexpr (GC == 2) dft<R, 1, 1, R>(v);
+#pragma unroll
+    for (int g = 0; g < GC; ++g)
+#pragma unroll
+        for (int c = 0; c < R; ++c) ex[(k1 + 16 * (hi + (NT / 16) * g) + 16 * Q * c) * CT + col] = v[g * R + c];
+    float2 w[8];
+#pragma unroll
+    for (int g = 0; g < GB; ++g)
+        twiddle_factors<Q>(L, 16 * (hi + (NT / 16) * g), [&](int i, int e) { w[g * (Q / 2) + i] = cconj(__ldg(&tw[e & MASK])); });
+    __syncthreads();
+#pragma unroll
+    for (int g = 0; g < GB; ++g) {
+#pragma unroll
+        for (int k2 = 0; k2 < Q; ++k2) v[g * Q + k2] = ex[(k1 + 16 * k2 + 16 * Q * (hi + (NT / 16) * g)) * CT + col];
+        dft_twiddled<Q>(v + g * Q, w + g * (Q / 2));
+    }
+    twiddle_factors<16>(L, t, [&](int i, int e) { w[i] = cconj(__ldg(&tw[e & MASK])); });
+    __syncthreads();
+#pragma unroll
+    for (int g = 0; g < GB; ++g)
+#pragma unroll
+        for (int b = 0; b < Q; ++b) ex[((b * R + hi + (NT / 16) * g) + LD * k1) * CT + col] = v[g * Q + b];
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < 16; ++k) v[k] = ex[(t + LD * k) * CT + col];
+    dft_twiddled<16>(v, w);
+}
+
 // Row pass, inverse, with the product: B[r][n2] = IFFT_P2 over k2 of X[r][.] * H[r][.].
+// Bound by memory latency (X from L2, H streamed from DRAM, B written): 32 us per 2^23-point
+// template against 50 us with two exchange buffers and 31 twiddle loads per thread.
 template <int P2>
 __global__ void __launch_bounds__(P2 / 16) fdfir_row_inv(const float2 *__restrict__ X, const float2 *__restrict__ H,
                                                          float2 *__restrict__ B, const float2 *__restrict__ tw2)
 {
     constexpr int NT2 = P2 / 16;
     extern __shared__ float2 fd_smem[];
-    float2 *e1 = fd_smem, *e2 = e1 + P2;
     const int tid = threadIdx.x;
-    const size_t off = (size_t)blockIdx.x * P2;
+    const size_t off = (size_t)blockIdx.x * P2 + tid;
     float2 v[16];
 #pragma unroll
-    for (int j = 0; j < 16; ++j) v[j] = cmul(__ldg(&X[off + j * NT2 + tid]), __ldg(&H[off + j * NT2 + tid]));
-    inverse_fft<P2>(v, e1, e2, tw2);
+    for (int j = 0; j < 16; ++j) v[j] = cmul(__ldg(&X[off + j * NT2]), __ldcs(&H[off + j * NT2]));
+    inverse_fft_folded<P2, 1>(v, fd_smem, tw2, tid, 0);
 #pragma unroll
-    for (int a = 0; a < 16; ++a) B[off + a * NT2 + tid] = v[a];
+    for (int a = 0; a < 16; ++a) B[off + a * NT2] = v[a];
 }
 
 // Column pass, inverse, with the power: out[P2 n1 + n2] = |IFFT_P1 over k1 of
 // W_P^{-n2 k1} B[r(k1)][n2]|^2 for P2 n1 + n2 < n.
-template <int P2>
-__global__ void __launch_bounds__(fd::NT1) fdfir_col_inv(const float2 *__restrict__ B, const float2 *__restrict__ tw1,
-                                                        float *__restrict__ out, int64_t n)
+//
+// CT columns at once: thread (t, column) with the column in the low bits of the thread index, so
+// that a row's CT values are read straight into registers as one contiguous run, all 16 loads of
+// a thread in flight, and the exchanges (values of the CT columns side by side, one buffer used
+// twice) are free of bank conflicts.  The twiddle of slot (g, k3) is a base per g times a step
+// per k3: two sincospif per thread and 8 per column.
+template <int P2, int CT>
+__global__ void __launch_bounds__(fd::NT1 *CT, 2) fdfir_col_inv(const float2 *__restrict__ B, const float2 *__restrict__ tw1,
+                                                               float *__restrict__ out, int64_t n)
 {
     using namespace fd;
-    extern __shared__ float2 fd_smem[];
-    float2 *tile = fd_smem, *e1 = tile + (size_t)P1 * TBP, *e2 = e1 + P1;
-    const int tid = threadIdx.x, n2_0 = blockIdx.x * TB;
+    constexpr int R = Geo<P1>::R, NT = NT1, LD = NT + 1;
+    static_assert(R == 8, "slots (g, k3) of the 2048-point transform");
     constexpr float two_over_p = 2.0f / ((float)P1 * (float)P2);
-    for (int idx = tid; idx < P1 * TB; idx += NT1) {
-        const int r = idx / TB, t = idx % TB;
-        tile[r * TBP + t] = B[(size_t)r * P2 + n2_0 + t];
+    extern __shared__ float2 fd_smem[];
+    float2 *ex = fd_smem, *step = fd_smem + (size_t)16 * LD * CT;
+    const int col = threadIdx.x % CT, t = threadIdx.x / CT, k1 = t & 15, hi = t >> 4;
+    const int n2 = blockIdx.x * CT + col;
+    float2 v[16];
+    const float2 *src = B + (size_t)t * P2 + n2;
+#pragma unroll
+    for (int j = 0; j < 16; ++j) v[j] = __ldg(src + (size_t)j * NT * P2);
+    if (t < 8) step[t * CT + col] = twiddle_p(n2 * 256 * t, two_over_p, 1.f);   // n2 k1 < 2^23
+    const float2 base0 = twiddle_p(n2 * (k1 + 16 * hi), two_over_p, 1.f);
+    const float2 base1 = twiddle_p(n2 * (k1 + 16 * (hi + NT / 16)), two_over_p, 1.f);
+    __syncthreads();
+#pragma unroll
+    for (int c = 0; c < R; ++c) {
+        const float2 s = step[c * CT + col];
+        v[c] = cmul(v[c], c == 0 ? base0 : cmul(base0, s));
+        v[R + c] = cmul(v[R + c], c == 0 ? base1 : cmul(base1, s));
     }
-    for (int t = 0; t < TB; ++t) {
-        __syncthreads();   // tile loaded; the previous column's exchanges are read
-        const int n2 = n2_0 + t;
-        float2 v[16];
+    inverse_fft_folded<P1, CT>(v, ex, tw1, t, col);
 #pragma unroll
-        for (int j = 0; j < 16; ++j) {
-            const int k1 = freq_of_slot(P1, tid, j);
-            v[j] = cmul(tile[(j * NT1 + tid) * TBP + t], twiddle_p(n2 * k1, two_over_p, 1.f));
-        }
-        inverse_fft<P1>(v, e1, e2, tw1);
-#pragma unroll
-        for (int a = 0; a < 16; ++a) {
-            const int64_t i = (int64_t)P2 * (a * NT1 + tid) + n2;
-            if (i < n) out[i] = cabs2(v[a]);
-        }
+    for (int a = 0; a < 16; ++a) {
+        const int64_t i = (int64_t)P2 * (a * NT + t) + n2;
+        if (i < n) out[i] = cabs2(v[a]);
     }
 }
 
@@ -165,14 +221,14 @@ static cudaError_t fdfir_attrs()
     e = cudaFuncSetAttribute(fdfir_col_fwd<P2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)fd::col_smem_bytes());
     if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(fdfir_col_inv<P2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)fd::col_smem_bytes());
+        e = cudaFuncSetAttribute(fdfir_col_inv<P2, fd::CT_INV>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)fd::col_inv_smem_bytes());
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(fdfir_row_fwd<P2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)fd::row_smem_bytes<P2>());
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(fdfir_row_inv<P2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)fd::row_smem_bytes<P2>());
+                                 (int)fd::row_inv_smem_bytes<P2>());
     if (e == cudaSuccess && dev >= 0 && dev < 64) done[dev] = true;
     return e;
 }
@@ -196,8 +252,8 @@ static cudaError_t fdfir_inverse_l(const float2 *X, const float2 *H, float2 *B, 
 {
     cudaError_t e = fdfir_attrs<P2>();
     if (e != cudaSuccess) return e;
-    fdfir_row_inv<P2><<<fd::P1, P2 / 16, fd::row_smem_bytes<P2>(), s>>>(X, H, B, tw2);
-    fdfir_col_inv<P2><<<P2 / fd::TB, fd::NT1, fd::col_smem_bytes(), s>>>(B, tw1, out, n);
+    fdfir_row_inv<P2><<<fd::P1, P2 / 16, fd::row_inv_smem_bytes<P2>(), s>>>(X, H, B, tw2);
+    fdfir_col_inv<P2, fd::CT_INV><<<P2 / fd::CT_INV, fd::NT1 * fd::CT_INV, fd::col_inv_smem_bytes(), s>>>(B, tw1, out, n);
     return cudaGetLastError();
 }
 

@@ -195,4 +195,57 @@ struct Dft<16, DIR, ST, OFF> {
 template <int R, int DIR, int ST = 1, int OFF = 0>
 __device__ __forceinline__ void dft(float2 *v) { detail::Dft<R, DIR, ST, OFF>::run(v); }
 
+// Butterfly a +- w b in six FMAs: p = a + w b, then a - w b = 2 a - p.
+__device__ __forceinline__ void bfly_w(float2 &a, float2 &b, float wx, float wy)
+{
+    const float px = fmaf(-wy, b.y, fmaf(wx, b.x, a.x)), py = fmaf(wy, b.x, fmaf(wx, b.y, a.y));
+    b = make_float2(fmaf(2.f, a.x, -px), fmaf(2.f, a.y, -py));
+    a = make_float2(px, py);
+}
+
+// Inverse DFT of twiddled inputs, y[a] = sum_k (w^k v[k]) exp(+2 pi i a k / N), N = 8 or 16, in place
+// on v[0 .. N-1], natural order in and out: radix-2 levels with the twiddles folded into the
+// butterflies, so N/2 factors are read instead of N - 1 twiddles.  The level that joins
+// sub-transforms at stride m takes the factors w^m exp(2 pi i u / N') before the quarter turn,
+// held in t in the order of twiddle_factors.
+template <int N>
+__device__ __forceinline__ void dft_twiddled(float2 *v, const float2 *t)
+{
+    int ti = 0;
+#pragma unroll
+    for (int m = N / 2; m >= 1; m /= 2) {
+        const int nu = N / (2 * m);                 // points at which the joined sub-transforms are known
+        const int nq = nu > 1 ? nu / 2 : 1;         // of them before the quarter turn
+        float2 o[N];
+#pragma unroll
+        for (int r = 0; r < m; ++r)
+#pragma unroll
+            for (int u = 0; u < nu; ++u) {
+                float2 a = v[r * nu + u], b = v[(r + m) * nu + u];   // k = r and r + m mod 2 m
+                const float2 w = t[ti + u % nq];
+                if (u < nq) bfly_w(a, b, w.x, w.y);
+                else bfly_w(a, b, -w.y, w.x);
+                o[r * 2 * nu + u] = a;
+                o[r * 2 * nu + u + nu] = b;
+            }
+#pragma unroll
+        for (int k = 0; k < N; ++k) v[k] = o[k];
+        ti += nq;
+    }
+}
+
+// The N/2 factors of dft_twiddled for w = exp(2 pi i e / L): set(i, exponent in units of 2 pi / L).
+template <int N, class F>
+__device__ __forceinline__ void twiddle_factors(int L, int e, F &&set)
+{
+    int ti = 0;
+#pragma unroll
+    for (int m = N / 2; m >= 1; m /= 2) {
+        const int nu = N / (2 * m), nq = nu > 1 ? nu / 2 : 1;
+#pragma unroll
+        for (int u = 0; u < nq; ++u) set(ti + u, m * e + u * (L / (2 * nu)));
+        ti += nq;
+    }
+}
+
 }  // namespace fdas
