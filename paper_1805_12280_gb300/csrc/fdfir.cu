@@ -20,6 +20,7 @@
 #include "fdas_internal.cuh"
 #include "fft_regs.cuh"
 #include "ols_common.cuh"
+#include "ptx.cuh"
 
 namespace fdas {
 
@@ -44,8 +45,6 @@ constexpr size_t row_smem_bytes()
 // where it touches the scratch B that the two passes hand back and forth.  A block of launch i
 // passes its wait before it ends, so the end of a launch implies the end of all before it.
 // 85 templates of 2^23 points: 5896 us without the overlap, 5046 with it (gaps and last waves).
-__device__ __forceinline__ void launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
-__device__ __forceinline__ void wait_prerequisites() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
 // exp(dir * 2 pi i e / P), e < P <= 2^23 (the argument 2e/P is exact in FP32)
 __device__ __forceinline__ float2 twiddle_p(int e, float two_over_p, float dir)
@@ -169,11 +168,11 @@ __global__ void __launch_bounds__(P2 / 16) fdfir_row_inv(const float2 *__restric
     const int tid = threadIdx.x;
     const size_t off = (size_t)blockIdx.x * P2 + tid;
     float2 v[16];
-    fd::launch_dependents();
+    launch_dependents();
 #pragma unroll
     for (int j = 0; j < 16; ++j) v[j] = cmul(__ldg(&X[off + j * NT2]), __ldcs(&H[off + j * NT2]));
     inverse_fft_folded<P2, 1>(v, fd_smem, tw2, tid, 0);
-    fd::wait_prerequisites();   // the column pass of the previous template has read B
+    wait_prerequisites();   // the column pass of the previous template has read B
 #pragma unroll
     for (int a = 0; a < 16; ++a) B[off + a * NT2] = v[a];
 }
@@ -198,7 +197,7 @@ __global__ void __launch_bounds__(fd::NT1 *CT, 2) fdfir_col_inv(const float2 *__
     float2 *ex = fd_smem, *step = fd_smem + (size_t)16 * LD * CT;
     const int col = threadIdx.x % CT, t = threadIdx.x / CT, k1 = t & 15, hi = t >> 4;
     const int n2 = blockIdx.x * CT + col;
-    fd::launch_dependents();
+    launch_dependents();
     if (t < 8) step[t * CT + col] = twiddle_p(n2 * 256 * t, two_over_p, 1.f);   // n2 k1 < 2^23
     const float2 base0 = twiddle_p(n2 * (k1 + 16 * hi), two_over_p, 1.f);
     const float2 base1 = twiddle_p(n2 * (k1 + 16 * (hi + NT / 16)), two_over_p, 1.f);

@@ -32,6 +32,7 @@
 #include <utility>
 
 #include "fdas_internal.cuh"
+#include "ptx.cuh"
 
 namespace fdas {
 namespace {
@@ -168,7 +169,7 @@ __global__ void __launch_bounds__(kHsThreads, 2) harmonic_kernel_narrow(const fl
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     // the next run of rows reads the same plane and appends to the same list: nothing here
     // feeds it, so it may start as soon as this launch's blocks leave room
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    launch_dependents();
     if (lane == 0) n_staged[warp] = 0;
     __syncwarp();
     const int c = (m - 1) / 2;
@@ -221,6 +222,9 @@ __global__ void __launch_bounds__(kHsThreads, 2) harmonic_kernel_narrow(const fl
     }
     __syncwarp();
     if (n_staged[warp]) warp_flush(stage[warp], &n_staged[warp], lane, out, max_cand, count);
+    // one block stays until the launch before has ended, so that the end of a launch stands for the
+    // end of all before it: a dependent launch that follows the last one may overwrite the plane
+    if (blockIdx.x == 0) wait_prerequisites();
 }
 
 using NarrowKernel = void (*)(const float *, int, int, int, int, int, int, HsThresholds, HsLimits,

@@ -107,8 +107,28 @@ struct Block {
     }
 };
 
+// Thread 0 of a one-item block: the first template(s), then, once the launch before is complete,
+// the segment into e1.
 template <int L>
-__device__ __forceinline__ void init_block(Block<L> &B, const OlsArgs &a)
+__device__ __forceinline__ void issue_loads(Block<L> &B, const OlsArgs &a, const CUtensorMap *map, int seg, int z0, int z1)
+{
+    constexpr int NT = Geo<L>::NT;
+    constexpr uint32_t HBYTES = (uint32_t)Smem<L>::h_bytes;
+    for (int i = 0; i < hbuf<L>() && z0 + i < z1; ++i) {
+        mbar_arrive_expect_tx(&B.bar[1 + i], HBYTES);
+        bulk_load(B.hb + i * 8 * NT, a.H + (size_t)(z0 + i) * 8 * NT, HBYTES, &B.bar[1 + i]);
+    }
+    wait_prerequisites();   // the input may come from the launch before; the templates are the plan's
+    mbar_arrive_expect_tx(&B.bar[0], (uint32_t)(L * sizeof(float2)));
+    const int c0 = seg * a.S - (a.K - 1);
+#pragma unroll
+    for (int j = 0; j < L / 256; ++j) tma_load_1d(B.e1 + 256 * j, map, c0 + 256 * j, &B.bar[0]);
+}
+
+// `first` runs in thread 0 as soon as the barriers are ready: the loads are in flight while the
+// block allocates tensor memory (warp AW: not thread 0's where `first` waits) and reads its twiddles.
+template <int L, int AW, class First>
+__device__ __forceinline__ void init_block(Block<L> &B, const OlsArgs &a, First first)
 {
     using Gm = Geo<L>;
     constexpr int NT = Gm::NT, Q = Gm::Q, R = Gm::R, GB = Gm::GB, GC = Gm::GC, MASK = L - 1;
@@ -118,8 +138,9 @@ __device__ __forceinline__ void init_block(Block<L> &B, const OlsArgs &a)
         mbar_init(&B.bar[1], 1);
         mbar_init(&B.bar[2], 1);
         fence_mbar_init();
+        first();
     }
-    if ((tid >> 5) == 0) tmem_alloc(B.tslot, kTmemCols<L>);
+    if ((tid >> 5) == AW) tmem_alloc(B.tslot, kTmemCols<L>);
     tmem_fence_before_sync();
     __syncthreads();
     tmem_fence_after_sync();
@@ -145,13 +166,13 @@ __device__ __forceinline__ void init_block(Block<L> &B, const OlsArgs &a)
 }
 
 // Every thread of the block, after its last TMEM access: the allocating warp frees it.
-template <int L>
+template <int L, int AW>
 __device__ __forceinline__ void release_block(Block<L> &B)
 {
     tmem_fence_before_sync();
     __syncthreads();
     tmem_fence_after_sync();
-    if ((threadIdx.x >> 5) == 0) tmem_dealloc(B.tmem, kTmemCols<L>);
+    if ((threadIdx.x >> 5) == AW) tmem_dealloc(B.tmem, kTmemCols<L>);
 }
 
 // After a timed-out wait: give each copy that may still be in flight a bounded time to
@@ -178,14 +199,16 @@ struct NoNext {
 // item is then called with `prefetched` set, transforms the segment from there and loads
 // its first template only after the forward pass A.
 //
-// VMASK: the plane stores test a bit mask of the thread's kept slots (per item; per template
-// near the array end for grouped plans) instead of comparing each output index: fewer instructions per
-// template in the one-item kernel; the persistent kernel, at its register limit, runs faster
-// without it.
-template <int L, bool CAND = false, class Next = NoNext, bool VMASK = false>
+// ONE: the one-item kernel.  Its loads are under way when run_item is called (issue_loads), the
+// block lets the next launch start when it begins its last template, and the plane stores
+// (VMASK) test a bit mask of the thread's kept slots (per item; per template near the array end for
+// grouped plans) instead of comparing each output index: fewer instructions per template; the
+// persistent kernel, at its register limit, runs faster without the mask.
+template <int L, bool CAND = false, class Next = NoNext, bool ONE = false>
 __device__ __forceinline__ bool run_item(Block<L> &B, const OlsArgs &a, const CUtensorMap *map, int seg, int z0,
                                          int z1, int64_t n, float *out, bool prefetched = false, Next next = Next())
 {
+    constexpr bool ISSUED = ONE, VMASK = ONE && !CAND;
     using Gm = Geo<L>;
     constexpr int NT = Gm::NT, Q = Gm::Q, R = Gm::R, GB = Gm::GB, GC = Gm::GC, LD2 = Gm::LD2;
     constexpr uint32_t HBYTES = (uint32_t)Smem<L>::h_bytes;
@@ -197,7 +220,7 @@ __device__ __forceinline__ bool run_item(Block<L> &B, const OlsArgs &a, const CU
 
     static_assert(NHB == 2 || HBYTES == L * sizeof(float2), "a prefetched segment fills the template buffer");
     static_assert(NHB == 2 || (sizeof(float2) * (L + 16 * Gm::LD2)) % 128 == 0, "TMA destination alignment");
-    if (tid == 0 && !prefetched) {
+    if (!ISSUED && tid == 0 && !prefetched) {
         fence_proxy_async_smem();   // earlier generic writes to e1/hb are ordered before the async copies
         mbar_arrive_expect_tx(&bar[0], (uint32_t)(L * sizeof(float2)));
         const int c0 = seg * a.S - (a.K - 1);
@@ -250,6 +273,7 @@ __device__ __forceinline__ bool run_item(Block<L> &B, const OlsArgs &a, const CU
     }
 
     for (int z = z0; z < z1; ++z) {
+        if (ONE && z + 1 == z1) launch_dependents();   // (see launch_lc)
         // output row and shift of this template (identity unless the plan groups templates)
         int row = z;
         int64_t shift = 0;
@@ -455,10 +479,11 @@ __global__ void __launch_bounds__(L / 16, MINB)
         B.sc = reinterpret_cast<unsigned *>(B.sb + kCandCap);
         if (threadIdx.x == 0) *B.sc = 0;
     }
-    init_block<L>(B, a);   // its barriers also publish *B.sc = 0
-    const int z0 = blockIdx.y * a.G;
-    run_item<L, CAND, NoNext, !CAND>(B, a, &tmap, a.seg_begin + blockIdx.x, z0, min(z0 + a.G, a.M), a.n, a.out);
-    release_block<L>(B);
+    const int seg = a.seg_begin + blockIdx.x, z0 = blockIdx.y * a.G, z1 = min(z0 + a.G, a.M);
+    init_block<L, 1>(B, a, [&]() { issue_loads(B, a, &tmap, seg, z0, z1); });   // its barriers also publish *B.sc = 0
+    wait_prerequisites();   // before any output is written
+    run_item<L, CAND, NoNext, true>(B, a, &tmap, seg, z0, z1, a.n, a.out);
+    release_block<L, 1>(B);
 }
 
 // Array of a batch item: the last array whose first item is <= item.
@@ -484,7 +509,7 @@ __global__ void __launch_bounds__(L / 16, MINB)
     extern __shared__ unsigned char smem_raw[];
     __shared__ int item_sh;
     Block<L> B(smem_raw);
-    init_block<L>(B, a);
+    init_block<L, 0>(B, a, []() {});
     if (threadIdx.x == 0) item_sh = atomicAdd(counter, 1);
     __syncthreads();
     int64_t item = item_sh;
@@ -510,7 +535,7 @@ __global__ void __launch_bounds__(L / 16, MINB)
         item = item_sh;
         prefetched = hbuf<L>() == 1 && item < tab.total_items;
     }
-    release_block<L>(B);
+    release_block<L, 0>(B);
 }
 
 template <int L>
@@ -537,9 +562,25 @@ static cudaError_t launch_lc(const CUtensorMap *tmap, const OlsArgs &a, int nseg
     static bool done[64] = {};
     cudaError_t e = set_smem_attr<L>((const void *)kern, done, smem);
     if (e != cudaSuccess) return e;
-    dim3 grid(nseg, (a.M + a.G - 1) / a.G);
-    kern<<<grid, L / 16, smem, s>>>(*tmap, a);
-    return cudaGetLastError();
+    // Programmatic dependent launch: blocks start, allocate their tensor memory and read their
+    // twiddles while the launch before drains, and wait for its end before they read the input or
+    // write the output.  A block lets the next launch start when it begins its last template: it
+    // holds its tensor memory then, so a block that waits never holds columns that the launch
+    // before still needs (and starts its dependents late enough: let go at its start, their blocks
+    // fill the SMs that drain first and run four to an SM beside idle ones, 32768 points in a graph
+    // 16.4 us against 12.8).  us per call, back to back, before and after: 16384 points 12.3 / 10.0,
+    // 65536 24.7 / 21.1, 301000 69.5 / 65.9, 2^22 722 / 720.
+    cudaLaunchAttribute attr{};
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(nseg, (a.M + a.G - 1) / a.G);
+    cfg.blockDim = dim3(L / 16);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kern, *tmap, a);
 }
 
 template <int L>

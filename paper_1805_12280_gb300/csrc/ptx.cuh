@@ -87,6 +87,12 @@ __device__ __forceinline__ void bulk_load(void *dst_smem, const void *src, uint3
         : "memory");
 }
 
+// Programmatic dependent launch.  launch_dependents lets the next launch on the stream start
+// once every block of this one has called it; wait_prerequisites returns when the launches
+// before are complete and their writes visible.
+__device__ __forceinline__ void launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void wait_prerequisites() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 // Status bits written by kernels into the plan's device status word.
 enum : int { STATUS_WAIT_TIMEOUT = 1 };
 
