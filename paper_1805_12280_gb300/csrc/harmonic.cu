@@ -9,30 +9,30 @@
 // is defined where |h z| <= c and bin0 + h r <= n - 1, and every S_h above its level's
 // threshold becomes a candidate.
 //
-// A thread takes Q fundamentals of one row, 256 apart (Q H = 64 for H >= 8, Q = 8 below):
-// all Q H loads of their harmonics are issued before the first is used (predicated on the
-// harmonic lying inside the plane), then each sum is formed in the order k = 1, 2, .., the
-// running sum compared with the threshold at every power of two.  A block takes tiles of
-// 256 Q consecutive fundamentals of one row (the k = 1 loads of a warp are one 128-byte
-// line; the k-th are a k-strided gather over k lines); in the 64-bit kernel its crossings
-// are staged per block and reserved in the output with one atomic per tile.  The kernel is bound by
-// instruction issue, so for planes narrower than 2^31 columns: rows are launched in runs of
-// equal kz = min(H, c / |z|) (the harmonics whose drift lies in the plane), each run by a
-// kernel compiled for exactly kz harmonics; each harmonic k has one base address per tile,
-// the thread's Q loads sit at fixed offsets 256 k q from it, and the test "bin0 + k r inside
-// the plane" is one 32-bit compare against r_lim[k] = (n-1-bin0)/k; crossings are staged per
-// warp, with no block barrier.
+// A thread takes Q fundamentals of one row, 256 apart: all loads of their harmonics are issued
+// before the first is used, then each sum is formed in the order k = 1, 2, .., the running sum
+// compared with the threshold at every power of two.  A block takes tiles of 256 Q consecutive
+// fundamentals of one row (the k = 1 loads of a warp are one 128-byte line; the k-th are a
+// k-strided gather over k lines).
+//
+// Planes narrower than 2^31 columns take one launch that walks the plane in slope windows (below)
+// with code compiled for each number of harmonics that lie in the plane; crossings are staged
+// per warp, with no block barrier.  85 x 2^22, 8 harmonics: 326 us, 1.44 GB read from DRAM (the
+// plane once), against 597 us and 3.40 GB when rows were launched in runs of equal harmonic
+// count and every strided pass fetched its rows again; 32 harmonics 842 -> 508 us, one harmonic
+// 272 -> 228 us, 65536 columns 61 -> 23 us per call (15 launches -> 1).  What bounds it: load
+// latency at 16 warps per SM (issue 40 %, DRAM 58 % of the measured copy rate); three blocks per SM
+// (fewer loads in flight per thread) are 6 % slower.
+// Wider rows (and more than 4097 of them) take the general kernel with 64-bit indexing.
 #include <cuda_runtime.h>
 
 #include <algorithm>
-#include <array>
+#include <atomic>
 #include <cstdint>
 #include <cstdio>
-#include <cstdlib>
-#include <utility>
+#include <type_traits>
 
 #include "fdas_internal.cuh"
-#include "ptx.cuh"
 
 namespace fdas {
 namespace {
@@ -151,102 +151,221 @@ __device__ __forceinline__ void warp_flush(fdas_harmonic_candidate *stage, unsig
     __syncwarp();
 }
 
-// One launch per run of rows with the same number KZ = min(H, c / |z|) of harmonics inside
-// the plane's drift range, compiled for exactly that many: no work on harmonics a row lacks.
-template <int KZ>
-__global__ void __launch_bounds__(kHsThreads, 2) harmonic_kernel_narrow(const float *__restrict__ P, int m, int n,
-                                                                        int bin0, int y0, int nrows, int tiles_per_row,
-                                                                        HsThresholds thr, HsLimits lim,
-                                                                        fdas_harmonic_candidate *__restrict__ out,
-                                                                        int64_t max_cand,
-                                                                        unsigned long long *__restrict__ count)
+// Slope windows.  Harmonic k of fundamental (r, z) lies in row k z at column k r: on the ray of
+// slope r / |z| through (c, bin0).  The cells of all rows with slopes in (S_w, S_{w+1}] are therefore
+// closed under the sums, and the plane is walked window by window: row |z| = a takes the
+// fundamentals (a S_w, a S_{w+1}], and every harmonic it reads lies in the part of row k a that the
+// same window reads as fundamentals, so all but the first read of a cell hit L2.  The z = 0 row
+// (its harmonics lie in itself) comes first.  Windows of 64 MB (8 harmonics at 2^22, sorted
+// records included: 16 MB 766, 32 MB 711, 64 MB 693, the whole plane 771 us in one version).
+constexpr int kHsMaxWin = 128, kHsMaxEntries = 2048;   // windows; (window, |z|) entries of one launch
+constexpr int64_t kHsWindowBytes = 64ll << 20;
+struct HsWindows {
+    int count;
+    int slope[kHsMaxWin + 1];
+};
+
+// Fundamentals per thread of rows with kz harmonics: 48 to 64 loads in flight, and a bit per
+// (fundamental, level) in one mask (16 and 8 fundamentals for kz = 1 and 2: 609 us against 510).
+__host__ __device__ constexpr int hs_q(int kz) { return kz == 1 ? 48 : kz == 2 ? 24 : kz == 3 ? 16 : kz <= 8 ? 8 : 64 / kz; }
+__host__ __device__ constexpr int hs_levels(int kz) { return kz < 2 ? 1 : 1 + hs_levels(kz / 2); }
+
+// One tile of 256 Q fundamentals r0 + threadIdx.x + 256 q <= rend of row z, compiled for
+// exactly the KZ harmonics that lie in the plane's drift range.  The straight-line part only
+// marks crossings in a mask; the few marked ones are appended by one short loop, so that the
+// bodies of all KZ stay small (with an append per sum the kernel was bound by instruction fetch).
+template <int KZ, int Q = hs_q(KZ)>
+__device__ __forceinline__ void hs_tile(const float *__restrict__ P, int c, int n, int bin0, int z, int r0, int rend,
+                                        const HsThresholds &thr, const HsLimits &lim, fdas_harmonic_candidate *stage,
+                                        unsigned *n_staged, fdas_harmonic_candidate *__restrict__ out, int64_t max_cand,
+                                        unsigned long long *__restrict__ count)
 {
-    constexpr int H = KZ;
-    constexpr int Q = hs_per_thread<H>();
-    constexpr int TILE = kHsThreads * Q;
+    constexpr int LV = hs_levels(KZ);
+    using Mask = std::conditional_t<(Q * LV > 32), uint64_t, uint32_t>;   // a bit per sum
+    constexpr int BITS = Q * LV > 32 ? 6 : 5;
+    const int rt = r0 + (int)threadIdx.x;
+    float v[Q][KZ];
+    Mask valid = ~Mask(0);   // bits of the sums that are defined
+    if (r0 + kHsThreads * Q - 1 <= min(lim.r_lim[KZ], rend)) {   // every harmonic of the tile lies in the plane
+#pragma unroll
+        for (int k = 1; k <= KZ; ++k) {
+            const float *base = P + ((int64_t)(c + k * z) * n + bin0 + (int64_t)k * rt);   // cell (c + k z, bin0 + k r)
+#pragma unroll
+            for (int q = 0; q < Q; ++q) v[q][k - 1] = __ldg(base + k * kHsThreads * q);
+        }
+    } else {
+        valid = 0;
+#pragma unroll
+        for (int k = 1; k <= KZ; ++k) {
+            const float *base = P + ((int64_t)(c + k * z) * n + bin0 + (int64_t)k * rt);
+            const int last = min(lim.r_lim[k], rend), in = last < rt ? 0 : min((last - rt) / kHsThreads + 1, Q);   // q < in
+#pragma unroll
+            for (int q = 0; q < Q; ++q) v[q][k - 1] = q < in ? __ldg(base + k * kHsThreads * q) : 0.f;
+            if ((k & (k - 1)) == 0) valid |= (Mask)(in >= 64 ? ~0ull : (1ull << in) - 1) << (Q * (31 - __clz(k)));
+        }
+    }
+    Mask mask = 0;
+#pragma unroll
+    for (int q = 0; q < Q; ++q) {
+        float acc = v[q][0];
+#pragma unroll
+        for (int k = 1; k <= KZ; ++k) {
+            if (k > 1) acc += v[q][k - 1];
+            if ((k & (k - 1)) == 0) {   // level h = k: the sum replaces its last term
+                const int j = 31 - __clz(k);
+                if (acc > thr.t[j]) mask |= Mask(1) << (Q * j + q);
+                v[q][k - 1] = acc;
+            }
+        }
+    }
+    mask &= valid;
+    while (mask) {
+        const int b = (BITS == 6 ? __ffsll((long long)mask) : __ffs((int)mask)) - 1, j = b / Q;
+        mask &= mask - 1;
+        float t[1 << BITS];   // the sums by bit, then a tree of selects on the bits of b
+#pragma unroll
+        for (int i = 0; i < (1 << BITS); ++i) t[i] = i < Q * LV ? v[i % Q][(1 << (i / Q < LV ? i / Q : 0)) - 1] : 0.f;
+#pragma unroll
+        for (int bit = 0; bit < BITS; ++bit) {
+            const bool up = (b >> bit) & 1;
+#pragma unroll
+            for (int i = 0; i < ((1 << BITS) >> (bit + 1)); ++i) t[i] = up ? t[2 * i + 1] : t[2 * i];
+        }
+        const float power = t[0];
+        fdas_harmonic_candidate rec;
+        rec.tpl = c + z;
+        rec.power = power;
+        rec.bin = bin0 + rt + (b - Q * j) * kHsThreads;
+        rec.nharm = 1 << j;
+        rec.reserved = 0;
+        const unsigned slot = atomicAdd(n_staged, 1u);
+        if (slot < (unsigned)kWarpStage) {
+            stage[slot] = rec;
+        } else {   // staging full: reserve this record on its own
+            const unsigned long long at = atomicAdd(count, 1ull);
+            if ((long long)at < max_cand) out[at] = rec;
+        }
+    }
+}
+
+// One harmonic (a plain threshold of the plane): no cell is read twice, tiles go row by row.
+// Q = 48 for planes that fill the GPU with such tiles, 8 below.
+template <int Q>
+__global__ void __launch_bounds__(kHsThreads, 2) harmonic_kernel_rows(const float *__restrict__ P, int c, int n, int bin0,
+                                                                      int tiles_per_row, HsThresholds thr, HsLimits lim,
+                                                                      fdas_harmonic_candidate *__restrict__ out,
+                                                                      int64_t max_cand,
+                                                                      unsigned long long *__restrict__ count)
+{
     __shared__ fdas_harmonic_candidate stage[kHsThreads / 32][kWarpStage];
     __shared__ unsigned n_staged[kHsThreads / 32];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    // the next run of rows reads the same plane and appends to the same list: nothing here
-    // feeds it, so it may start as soon as this launch's blocks leave room
-    launch_dependents();
     if (lane == 0) n_staged[warp] = 0;
     __syncwarp();
-    const int c = (m - 1) / 2;
-    const int64_t tiles = (int64_t)nrows * tiles_per_row;
+    const int64_t tiles = (int64_t)(2 * c + 1) * tiles_per_row;
     for (int64_t tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
-        const int yr = (int)(tile / tiles_per_row);
-        const int y = y0 + yr;
-        const int z = y - c;
-        const int r0 = 1 + (int)(tile - (int64_t)yr * tiles_per_row) * TILE + (int)threadIdx.x;
-        float v[Q][H];
-#pragma unroll
-        for (int k = 1; k <= H; ++k) {
-            // cell (c + k z, bin0 + k r0); read only where the harmonic lies in the plane
-            const float *base = P + ((int64_t)(c + k * z) * n + bin0 + (int64_t)k * r0);
-#pragma unroll
-            for (int q = 0; q < Q; ++q) {
-                const bool in = r0 + q * kHsThreads <= lim.r_lim[k];
-                v[q][k - 1] = in ? __ldg(base + k * kHsThreads * q) : 0.f;
-            }
-        }
-#pragma unroll
-        for (int q = 0; q < Q; ++q) {
-            const int r = r0 + q * kHsThreads;
-            float acc = 0.f;
-#pragma unroll
-            for (int k = 1; k <= H; ++k) {
-                acc += v[q][k - 1];
-                if ((k & (k - 1)) == 0) {   // level h = k
-                    const int j = 31 - __clz(k);
-                    if (r <= lim.r_lim[k] && acc > thr.t[j]) {
-                        fdas_harmonic_candidate rec;
-                        rec.tpl = y;
-                        rec.power = acc;
-                        rec.bin = bin0 + r;
-                        rec.nharm = k;
-                        rec.reserved = 0;
-                        const unsigned slot = atomicAdd(&n_staged[warp], 1u);
-                        if (slot < (unsigned)kWarpStage) {
-                            stage[warp][slot] = rec;
-                        } else {   // staging full: reserve this record on its own
-                            const unsigned long long at = atomicAdd(count, 1ull);
-                            if ((long long)at < max_cand) out[at] = rec;
-                        }
-                    }
-                }
-            }
-        }
+        const int y = (int)(tile / tiles_per_row), first = 1 + (int)(tile - (int64_t)y * tiles_per_row) * kHsThreads * Q;
+        hs_tile<1, Q>(P, c, n, bin0, y - c, first, lim.r_lim[1], thr, lim, stage[warp], &n_staged[warp], out, max_cand, count);
         __syncwarp();
         if (n_staged[warp] >= (unsigned)kWarpFlush) warp_flush(stage[warp], &n_staged[warp], lane, out, max_cand, count);
     }
     __syncwarp();
     if (n_staged[warp]) warp_flush(stage[warp], &n_staged[warp], lane, out, max_cand, count);
-    // one block stays until the launch before has ended, so that the end of a launch stands for the
-    // end of all before it: a dependent launch that follows the last one may overwrite the plane
-    if (blockIdx.x == 0) wait_prerequisites();
 }
 
-using NarrowKernel = void (*)(const float *, int, int, int, int, int, int, HsThresholds, HsLimits,
-                              fdas_harmonic_candidate *, int64_t, unsigned long long *);
-
-template <int... K>
-constexpr std::array<NarrowKernel, sizeof...(K)> narrow_table(std::integer_sequence<int, K...>)
+template <int H>
+__global__ void __launch_bounds__(kHsThreads, 2) harmonic_kernel_slope(const float *__restrict__ P, int c, int n, int bin0,
+                                                                       HsThresholds thr, HsLimits lim, HsWindows win,
+                                                                       fdas_harmonic_candidate *__restrict__ out,
+                                                                       int64_t max_cand,
+                                                                       unsigned long long *__restrict__ count)
 {
-    return {&harmonic_kernel_narrow<K + 1>...};
+    __shared__ fdas_harmonic_candidate stage[kHsThreads / 32][kWarpStage];
+    __shared__ unsigned n_staged[kHsThreads / 32];
+    extern __shared__ int4 ent[];   // entry (window, |z| = c .. 1): its end in tiles, first and last
+                                    // fundamental, |z| << 14 | fundamentals per thread << 6 | harmonics
+    __shared__ int part[kHsThreads / 32];
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int rmax = lim.r_lim[1], entries = win.count * c;
+    {   // tile counts: each thread sums a run of entries, then a block scan
+        const int per = (entries + kHsThreads - 1) / kHsThreads, e0 = min(tid * per, entries), e1 = min(e0 + per, entries);
+        int sum = 0;
+        for (int e = e0; e < e1; ++e) {
+            const int w = e / c, a = c - (e - w * c);
+            const int64_t lo = (int64_t)a * win.slope[w], hi = (int64_t)a * win.slope[w + 1];
+            const int first = (int)(lo < rmax ? lo : rmax) + 1, last = (int)(hi < rmax ? hi : rmax);
+            // the harmonics of its first fundamental inside the plane (rows and columns)
+            const int kz = max(1, min(min(H, c / a), rmax / first)), tile = kHsThreads * hs_q(kz);
+            sum += 2 * ((last - first + tile) / tile);   // both signs of z
+            ent[e] = make_int4(sum, first, last, (a << 14) | (hs_q(kz) << 6) | kz);
+        }
+        int incl = sum;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int v = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= o) incl += v;
+        }
+        if (lane == 31) part[warp] = incl;
+        if (lane == 0) n_staged[warp] = 0;
+        __syncthreads();
+        int before = incl - sum;
+        for (int i = 0; i < warp; ++i) before += part[i];
+        for (int e = e0; e < e1; ++e) ent[e].x += before;
+        __syncthreads();
+    }
+    constexpr int TILE0 = kHsThreads * hs_q(H);
+    const int tiles0 = (rmax + TILE0 - 1) / TILE0;   // of the z = 0 row
+    const int tiles = tiles0 + (entries ? ent[entries - 1].x : 0);
+    int e = 0, begin = 0;   // the entry of this block's tile, and its first tile
+    for (int tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
+        int z = 0, kz = H, first = 1 + tile * TILE0, last = rmax;
+        if (tile >= tiles0) {
+            const int t = tile - tiles0;
+            int4 en = ent[e];
+            while (t >= en.x) {
+                begin = en.x;
+                en = ent[++e];
+            }
+            const int local = t - begin, half = (en.x - begin) >> 1;
+            kz = en.w & 63;
+            z = local < half ? en.w >> 14 : -(en.w >> 14);
+            first = en.y + (local < half ? local : local - half) * kHsThreads * ((en.w >> 6) & 255);
+            last = en.z;
+        }
+#define FDAS_HS_CASE(K)                                                                                                   \
+    case K:                                                                                                                \
+        if constexpr (K <= H)                                                                                              \
+            hs_tile<K>(P, c, n, bin0, z, first, last, thr, lim, stage[warp], &n_staged[warp], out, max_cand, count);       \
+        break;
+        switch (kz) {
+            FDAS_HS_CASE(1) FDAS_HS_CASE(2) FDAS_HS_CASE(3) FDAS_HS_CASE(4) FDAS_HS_CASE(5) FDAS_HS_CASE(6) FDAS_HS_CASE(7)
+            FDAS_HS_CASE(8) FDAS_HS_CASE(9) FDAS_HS_CASE(10) FDAS_HS_CASE(11) FDAS_HS_CASE(12) FDAS_HS_CASE(13)
+            FDAS_HS_CASE(14) FDAS_HS_CASE(15) FDAS_HS_CASE(16) FDAS_HS_CASE(17) FDAS_HS_CASE(18) FDAS_HS_CASE(19)
+            FDAS_HS_CASE(20) FDAS_HS_CASE(21) FDAS_HS_CASE(22) FDAS_HS_CASE(23) FDAS_HS_CASE(24) FDAS_HS_CASE(25)
+            FDAS_HS_CASE(26) FDAS_HS_CASE(27) FDAS_HS_CASE(28) FDAS_HS_CASE(29) FDAS_HS_CASE(30) FDAS_HS_CASE(31)
+            FDAS_HS_CASE(32)
+        }
+#undef FDAS_HS_CASE
+        __syncwarp();
+        if (n_staged[warp] >= (unsigned)kWarpFlush) warp_flush(stage[warp], &n_staged[warp], lane, out, max_cand, count);
+    }
+    __syncwarp();
+    if (n_staged[warp]) warp_flush(stage[warp], &n_staged[warp], lane, out, max_cand, count);
 }
 
-// harmonic_kernel_narrow<KZ> for KZ = 1 .. 32
-constexpr std::array<NarrowKernel, 32> kNarrow = narrow_table(std::make_integer_sequence<int, 32>{});
-
-cudaError_t resident_grid(const void *fn, int64_t tiles, unsigned *grid)
+// Blocks of `fn` that are resident at once (at most `tiles`); asked for once per kernel and device.
+cudaError_t resident_grid(const void *fn, int64_t tiles, size_t smem, std::atomic<int> (&known)[64], unsigned *grid)
 {
     int dev = 0, sms = 0, per_sm = 0;
     cudaError_t e;
     if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
-    if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
-    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, kHsThreads, 0)) != cudaSuccess) return e;
-    const int64_t resident = (int64_t)sms * (per_sm > 0 ? per_sm : 1);
+    int resident = dev >= 0 && dev < 64 ? known[dev].load(std::memory_order_relaxed) : 0;
+    if (!resident) {
+        if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
+        if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, kHsThreads, smem)) != cudaSuccess) return e;
+        resident = sms * (per_sm > 0 ? per_sm : 1);
+        if (dev >= 0 && dev < 64) known[dev].store(resident, std::memory_order_relaxed);
+    }
     *grid = (unsigned)(tiles < resident ? tiles : resident);
     return cudaSuccess;
 }
@@ -259,37 +378,53 @@ cudaError_t launch_hs(int H, const float *P, int m, int64_t n, int64_t bin0, con
     cudaError_t e;
     unsigned grid = 0;
     // 32-bit fundamentals and bins, with room for the last tile's overhang past rmax
-    if (n <= (((int64_t)1 << 31) - ((int64_t)1 << 16))) {
+    if (n <= (((int64_t)1 << 31) - ((int64_t)1 << 16)) && c <= kHsMaxEntries) {
         HsLimits lim{};
         for (int k = 1; k <= 32; ++k) lim.r_lim[k] = (int)(rmax / k);
-        auto kz_of = [&](int y) { const int az = std::abs(y - c); return az == 0 ? H : std::min(H, c / az); };
-        for (int y0 = 0; y0 < m;) {   // runs of rows with the same kz
-            const int kz = kz_of(y0);
-            int y1 = y0 + 1;
-            while (y1 < m && kz_of(y1) == kz) ++y1;
-            const NarrowKernel fn = kNarrow[kz - 1];
-            const int64_t tile = (int64_t)kHsThreads * (kz <= 8 ? 8 : 64 / kz);   // hs_per_thread<kz>()
-            const int64_t tiles_per_row = (rmax + tile - 1) / tile;
-            if ((e = resident_grid((const void *)fn, (int64_t)(y1 - y0) * tiles_per_row, &grid)) != cudaSuccess)
-                return e;
-            // launches after the first may overlap the one before (programmatic dependent launch):
-            // the runs are independent, and the tail of one run fills with the next
-            cudaLaunchAttribute attr{};
-            attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-            attr.val.programmaticStreamSerializationAllowed = 1;
-            cudaLaunchConfig_t cfg{};
-            cfg.gridDim = dim3(grid);
-            cfg.blockDim = dim3(kHsThreads);
-            cfg.dynamicSmemBytes = 0;
-            cfg.stream = s;
-            cfg.attrs = &attr;
-            cfg.numAttrs = y0 > 0 ? 1 : 0;
-            if ((e = cudaLaunchKernelEx(&cfg, fn, P, m, (int)n, (int)bin0, y0, y1 - y0, (int)tiles_per_row, thr, lim, out,
-                                        max_cand, count)) != cudaSuccess)
-                return e;
-            y0 = y1;
+        if (H == 1) {
+            static std::atomic<int> known[2][64];
+            const auto large = harmonic_kernel_rows<hs_q(1)>, small = harmonic_kernel_rows<8>;
+            const int64_t tile = (int64_t)kHsThreads * hs_q(1), per_row = (rmax + tile - 1) / tile;
+            if ((e = resident_grid((const void *)large, (int64_t)m * per_row, 0, known[0], &grid)) != cudaSuccess) return e;
+            if ((int64_t)m * per_row > 2 * (int64_t)grid) {
+                large<<<grid, kHsThreads, 0, s>>>(P, c, (int)n, (int)bin0, (int)per_row, thr, lim, out, max_cand, count);
+            } else {
+                const int64_t per_row8 = (rmax + kHsThreads * 8 - 1) / (kHsThreads * 8);
+                if ((e = resident_grid((const void *)small, (int64_t)m * per_row8, 0, known[1], &grid)) != cudaSuccess) return e;
+                small<<<grid, kHsThreads, 0, s>>>(P, c, (int)n, (int)bin0, (int)per_row8, thr, lim, out, max_cand, count);
+            }
+            return cudaGetLastError();
         }
-        return cudaSuccess;
+        HsWindows win{};
+        // windows of about kHsWindowBytes of the plane: rows |z| <= rmax / S reach slope S
+        int64_t S = 0, bytes = kHsWindowBytes;
+        const int most = c > 0 ? std::min(kHsMaxWin, kHsMaxEntries / c) : 1;
+        const int64_t plane = (int64_t)m * n * 4;
+        if (plane / most > bytes) bytes = plane / most;
+        while (S < rmax && c > 0) {
+            const int64_t a = std::min<int64_t>(c, S > 0 ? rmax / S : c);
+            S += std::max<int64_t>(1, bytes / (4 * a * (a + 1)));
+            if (win.count == most - 1 || S > rmax) S = rmax;
+            win.slope[++win.count] = (int)S;
+        }
+        using Kernel = void (*)(const float *, int, int, int, HsThresholds, HsLimits, HsWindows, fdas_harmonic_candidate *,
+                                int64_t, unsigned long long *);
+        Kernel fn;
+        switch (H) {
+        case 2: fn = harmonic_kernel_slope<2>; break;
+        case 4: fn = harmonic_kernel_slope<4>; break;
+        case 8: fn = harmonic_kernel_slope<8>; break;
+        case 16: fn = harmonic_kernel_slope<16>; break;
+        default: fn = harmonic_kernel_slope<32>; break;
+        }
+        // at most one tile per block: both signs of every row, its ragged ends, and the z = 0 row
+        const int64_t tiles = (int64_t)m * (rmax / kHsThreads + 1) + 2 * (int64_t)c * win.count;
+        // (the occupancy of the largest table, so that one number serves every call)
+        static std::atomic<int> known[6][64];
+        const int level = 31 - __builtin_clz((unsigned)H);
+        if ((e = resident_grid((const void *)fn, tiles, sizeof(int4) * kHsMaxEntries, known[level], &grid)) != cudaSuccess) return e;
+        fn<<<grid, kHsThreads, sizeof(int4) * (size_t)(win.count * c), s>>>(P, c, (int)n, (int)bin0, thr, lim, win, out, max_cand, count);
+        return cudaGetLastError();
     }
     const void *fn = nullptr;
     int64_t tile = 0;
@@ -302,7 +437,8 @@ cudaError_t launch_hs(int H, const float *P, int m, int64_t n, int64_t bin0, con
     default: fn = (const void *)harmonic_kernel<32>; tile = kHsThreads * hs_per_thread<32>(); break;
     }
     const int64_t tiles_per_row = (rmax + tile - 1) / tile;
-    if ((e = resident_grid(fn, (int64_t)m * tiles_per_row, &grid)) != cudaSuccess) return e;
+    static std::atomic<int> known[6][64];
+    if ((e = resident_grid(fn, (int64_t)m * tiles_per_row, 0, known[31 - __builtin_clz((unsigned)H)], &grid)) != cudaSuccess) return e;
     switch (H) {
     case 1: harmonic_kernel<1><<<grid, kHsThreads, 0, s>>>(P, m, n, bin0, tiles_per_row, thr, out, max_cand, count); break;
     case 2: harmonic_kernel<2><<<grid, kHsThreads, 0, s>>>(P, m, n, bin0, tiles_per_row, thr, out, max_cand, count); break;
