@@ -36,6 +36,7 @@
 #include <cuda_runtime.h>
 
 #include <cmath>
+#include <type_traits>
 
 #include "fdas_internal.cuh"
 #include "fft_regs.cuh"
@@ -640,6 +641,13 @@ __device__ __forceinline__ void tc2_body(const Src &src, const tc2::Args &a)
             __syncwarp();
             nst = 0;
         };
+        // The runs n2 < (K - 1) / 32 lie wholly in the discarded K - 1 outputs (13 of the 64 at K = 421).
+        // SKIP: they are neither loaded nor squared, as far as whole chunks of 16 runs or the first
+        // 12 of a chunk go (85 templates, K = 421: 2^22 points 424 -> 420 us, 24 arrays of 2^18 to 2^22
+        // points 2932 -> 2887).  Not for short arrays, where the longer code costs more (65536 points
+        // 14.8 -> 15.5 us), nor for thresholds, where it gave nothing.
+        constexpr bool SKIP = !CAND && !std::is_same_v<Src, SingleGroupSrc>;
+        const int run0 = (a.K - 1) >> 5, first_n2 = (run0 & 15) >= 12 ? (run0 & ~15) + 12 : run0 & ~15;
         uint32_t p = 0;
         int il = 0;
         for (int k = 0; k < nk; ++k, ++il) {
@@ -664,8 +672,32 @@ __device__ __forceinline__ void tc2_body(const Src &src, const tc2::Args &a)
                 tmem_fence_after_sync();
                 const int z = 2 * zp + zq;
                 float *o = ii.out + (size_t)z * (size_t)ii.n + segrow;
+                int cc = 0;
+                if constexpr (SKIP) {   // the last 4 runs of the first chunk, or from its start
+                    cc = first_n2 >> 4;
+                    if ((first_n2 & 15) == 12) {
+                        uint32_t r[8];
+                        tmem_ld8(my + 128 * (p & 1) + 2 * first_n2, r);
+                        if (cc == 3) {
+                            tmem_fence_before_sync();
+                            nb_arrive(NB_D2 + (p & 1));
+                        }
+                        if (z < a.M) {
+#pragma unroll
+                            for (int g = 0; g < 2; ++g) {
+                                const float2 re = make_float2(__uint_as_float(r[4 * g]), __uint_as_float(r[4 * g + 1]));
+                                const float2 im = make_float2(__uint_as_float(r[4 * g + 2]), __uint_as_float(r[4 * g + 3]));
+                                const float2 pw = pmul(pfma(re, re, pmul(im, im)), make_float2(fs, fs));
+                                const int t0 = tbase + 32 * (first_n2 + 2 * g);
+                                if ((unsigned)t0 < (unsigned)lim) o[t0] = pw.x;
+                                if ((unsigned)(t0 + 32) < (unsigned)lim) o[t0 + 32] = pw.y;
+                            }
+                        }
+                        ++cc;
+                    }
+                }
 #pragma unroll 1
-                for (int cc = 0; cc < 4; ++cc) {   // n2 = 16 cc .. 16 cc + 15
+                for (; cc < 4; ++cc) {   // n2 = 16 cc .. 16 cc + 15
                     uint32_t r[32];
                     tmem_ld32(my + 128 * (p & 1) + 32 * cc, r);
                     if (cc == 3) {
