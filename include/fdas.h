@@ -269,14 +269,15 @@ int fdas_selftest_wait_timeout(fdas_plan p, double limit_ms, void *stream);
  * alternative the paper weighs overlap-save against: y_z = IFFT_P(FFT_P(x) . FFT_P(h_z)) with
  * P the smallest power of two >= n_max + tpl_len - 1 (at least 2^21, at most 2^23), then
  * |y_z[i]|^2 for i < n -- the same plane as fdas_convolve (Eq. 1), computed with P-point
- * transforms of the whole array (four-step, P = 2048 x P/2048) instead of segments.
+ * transforms of the whole array (four-step, P = 1024 x P/1024) instead of segments.
  *
  * fdas_fdfir_create: synchronous; copies the M x K complex64 templates (host, row-major) and
  *   stores their P-point spectra on the current device (M x P x 8 bytes: 5.7 GB for 85
- *   templates at P = 2^23).  Errors: INVALID_ARG (null pointers, sizes < 1, n_max + tpl_len - 1
+ *   templates at P = 2^23; three more arrays of P values for a call's spectrum and
+ *   intermediate results).  Errors: INVALID_ARG (null pointers, sizes < 1, n_max + tpl_len - 1
  *   > 2^23), OOM, CUDA.
  * fdas_fdfir_length: *P = the transform length.
- * fdas_fdfir_convolve: enqueues on `stream` (2 + 2M kernel launches) the plane out[z][i]
+ * fdas_fdfir_convolve: enqueues on `stream` (3 + M kernel launches) the plane out[z][i]
  *   (float32, [M][n] row-major, device) of in[0, n) (complex64, device, 8-byte aligned);
  *   1 <= n <= n_max; in and out must not overlap.  Calls on one plan share its scratch and
  *   must not overlap on the GPU.  Errors: INVALID_ARG, CUDA.

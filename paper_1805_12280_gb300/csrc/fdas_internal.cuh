@@ -155,13 +155,16 @@ cudaError_t launch_td_direct(const float2 *x, int64_t n, const float2 *h, int M,
 
 // Plan-time kernels (FP64).
 cudaError_t launch_twiddles(int L, double2 *w64, float2 *w32, cudaStream_t s);
-// Full-length FD-FIR passes (P = 2048 * P2): forward transform of in[0, len) into A (times
-// scale); inverse of X . H into the power row out[0, n) through the scratch B (first: the launch
-// before on the stream is not an inverse of the same call; up: the direction of the row pass).
-cudaError_t fdfir_forward(int P2, const float2 *in, int64_t len, const float2 *tw1, const float2 *tw2, float2 *A,
-                          float scale, cudaStream_t s);
-cudaError_t fdfir_inverse(int P2, const float2 *X, const float2 *H, float2 *B, const float2 *tw1, const float2 *tw2,
-                          float *out, int64_t n, bool first, bool up, cudaStream_t s);
+// Full-length FD-FIR (P = 1024 * P2): forward transform of in[0, len) into A (times scale);
+// inverses of X . H_z into the power rows out[z][0, n) through the scratch B of 2 P values.  Tables:
+// w1 = W_1024; w2 = W_N of the in-block row transform, N = min(P2, 4096), then the N / 2 factors of
+// its last pass; wr = W_P2.
+struct FdfirTables {
+    const float2 *w1, *w2, *wr;
+};
+cudaError_t fdfir_forward(int P2, const float2 *in, int64_t len, const FdfirTables &tw, float2 *A, float scale, cudaStream_t s);
+cudaError_t fdfir_inverse(int P2, const float2 *X, const float2 *H, int M, float2 *B, const FdfirTables &tw, float *out,
+                          int64_t n, cudaStream_t s);
 // split: the slot pairs (c, 8 + c) as (re_c, re_{8+c}, im_c, im_{8+c}) (tensor-core form),
 // else the slot pairs (2p, 2p + 1) as two complex values.
 cudaError_t launch_pretransform(int L, const float2 *h32, int M, int K, const double2 *w64,
