@@ -56,7 +56,9 @@ typedef struct {
     int seg_len;      /* L, the overlap-save FFT length: 1024, 2048 or 4096 (0 = 2048) */
     int tpl_per_cta;  /* G, templates per thread block: 1..M; 0 = chosen per call from the number
                          of segments (all M for long arrays, fewer per block for short ones so
-                         that the launch still fills the GPU; the tensor-core form uses all M) */
+                         that the launch still fills the GPU; equal shares of the launch's work,
+                         across segments, where that is the faster split of a plane; the
+                         tensor-core form uses all M) */
     int precision;    /* FDAS_PREC_* (0 = FP32) */
     int autotune;     /* 1: time every (L in {1024, 2048, 4096}) x (G chosen per call, 5, 17, 85)
                          with the persistent batch kernel on a seeded proxy of the batches the
@@ -117,7 +119,8 @@ int fdas_plan_describe(fdas_plan p, fdas_plan_desc *desc);
 
 /* Templates per thread block that fdas_convolve uses for an array of n points (the plan's
  * fixed G, or the per-call choice when the plan was created with tpl_per_cta = 0; a grouped
- * plan applies the same rule to each template group and its segment count).
+ * plan applies the same rule to each template group and its segment count; where the blocks of
+ * a plane's launch take equal shares of its work instead, this is what the rule would have been).
  * Returns G >= 1, or a negative error code (INVALID_ARG for a null plan or n outside
  * [1, n_max]).  Host only; no CUDA call. */
 int fdas_plan_tpl_per_cta(fdas_plan p, int64_t n);

@@ -193,6 +193,23 @@ int call_G(const fdas_plan p, int64_t nseg, int m)
     return (m + ng - 1) / ng;
 }
 
+// Blocks that share the (segment, template) units of a one-array FP32 plane launch equally, one
+// wave of them, or 0: blocks of whole template groups (call_G).  Groups leave the last wave of
+// blocks partly empty; a share costs one more forward FFT where it crosses a segment boundary.
+// Measured over 21 lengths each at 6 to 63 units per block and 85, 43 and 21 templates, time of
+// shares / groups: from 7 units on, L = 4096 0.80 .. 0.99 and L = 1024 0.82 .. 0.96 at all sizes
+// (85 templates of 2^22 points 818 -> 756 us, 1060 -> 1038), L = 2048 0.91 .. 1.02 up to 45 units
+// (301000 points 66.0 -> 63.3 us, 400000 88.8 -> 81.7).  Below 7 units a share is too short for its
+// forward FFTs (41000 points 13.0 us against 15.6); longer ones with L = 2048, four blocks of four
+// warps an SM, drift apart and the last runs alone (2^22 points 721 us against 770), where groups
+// in several waves even out.  With 9 templates, 0.88 .. 1.09: groups.
+int call_blocks(fdas_plan p, int64_t nseg, int m, bool cand)
+{
+    if (!p->g_auto || cand || p->precision != FDAS_PREC_FP32 || m < 20) return 0;
+    const int64_t units = nseg * m, slots = p->bk.resident;
+    return units >= 7 * slots && (p->L != 2048 || units <= 45 * slots) ? p->bk.resident : 0;
+}
+
 fdas::OlsArgs base_args(fdas_plan p, int64_t n, float *out)
 {
     fdas::OlsArgs a;
@@ -213,6 +230,7 @@ fdas::OlsArgs base_args(fdas_plan p, int64_t n, float *out)
 int launch_range(fdas_plan p, const CUtensorMap *map, fdas::OlsArgs a, int64_t s0, int64_t s1, cudaStream_t stream)
 {
     a.seg_begin = (int)s0;
+    a.blocks = call_blocks(p, s1 - s0, a.M, a.cand != nullptr);
     cudaError_t e = fdas::launch_ols_fp32(p->L, map, a, (int)(s1 - s0), stream);
     if (e != cudaSuccess) return cuda_fail(e, "segment kernel launch");
     return FDAS_OK;
@@ -234,6 +252,7 @@ int launch_all(fdas_plan p, const CUtensorMap *map, const fdas::OlsArgs &a0, int
         const int64_t span = n - gr.min_shift;
         const int64_t nseg = span > 0 ? (span + gr.S - 1) / gr.S : 1;   // one segment writes the zero prefix
         a.G = call_G(p, nseg, gr.count);
+        a.blocks = call_blocks(p, nseg, gr.count, a.cand != nullptr);
         cudaError_t e = fdas::launch_ols_fp32(p->L, map, a, (int)nseg, stream);
         if (e != cudaSuccess) return cuda_fail(e, "segment kernel launch (template group)");
     }

@@ -65,6 +65,7 @@ struct OlsArgs {
     const unsigned char *H16 = nullptr;
     const unsigned char *cst = nullptr;
     int eH = 0, ng = 1;
+    int blocks = 0;       // FP32 form: blocks that share the launch's units equally (0: whole groups)
 };
 
 // One array of a batch: its input tensor map (param space), output plane and work items.

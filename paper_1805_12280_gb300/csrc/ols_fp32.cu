@@ -199,16 +199,18 @@ struct NoNext {
 // item is then called with `prefetched` set, transforms the segment from there and loads
 // its first template only after the forward pass A.
 //
-// ONE: the one-item kernel.  Its loads are under way when run_item is called (issue_loads), the
-// block lets the next launch start when it begins its last template, and the plane stores
-// (VMASK) test a bit mask of the thread's kept slots (per item; per template near the array end for
-// grouped plans) instead of comparing each output index: fewer instructions per template; the
-// persistent kernel, at its register limit, runs faster without the mask.
+// ONE: the one-array kernels.  The first item's loads are under way when run_item is called
+// (`issued`, see issue_loads), the block lets the next launch start when it begins the last
+// template of its `last` item, and the plane stores (VMASK) test a bit mask of the thread's kept
+// slots (per item; per template near the array end for grouped plans) instead of comparing each
+// output index: fewer instructions per template; the persistent kernel, at its register limit,
+// runs faster without the mask.
 template <int L, bool CAND = false, class Next = NoNext, bool ONE = false>
 __device__ __forceinline__ bool run_item(Block<L> &B, const OlsArgs &a, const CUtensorMap *map, int seg, int z0,
-                                         int z1, int64_t n, float *out, bool prefetched = false, Next next = Next())
+                                         int z1, int64_t n, float *out, bool prefetched = false, Next next = Next(),
+                                         bool issued = ONE, bool last = true)
 {
-    constexpr bool ISSUED = ONE, VMASK = ONE && !CAND;
+    constexpr bool VMASK = ONE && !CAND;
     using Gm = Geo<L>;
     constexpr int NT = Gm::NT, Q = Gm::Q, R = Gm::R, GB = Gm::GB, GC = Gm::GC, LD2 = Gm::LD2;
     constexpr uint32_t HBYTES = (uint32_t)Smem<L>::h_bytes;
@@ -220,7 +222,7 @@ __device__ __forceinline__ bool run_item(Block<L> &B, const OlsArgs &a, const CU
 
     static_assert(NHB == 2 || HBYTES == L * sizeof(float2), "a prefetched segment fills the template buffer");
     static_assert(NHB == 2 || (sizeof(float2) * (L + 16 * Gm::LD2)) % 128 == 0, "TMA destination alignment");
-    if (!ISSUED && tid == 0 && !prefetched) {
+    if (!issued && tid == 0 && !prefetched) {
         fence_proxy_async_smem();   // earlier generic writes to e1/hb are ordered before the async copies
         mbar_arrive_expect_tx(&bar[0], (uint32_t)(L * sizeof(float2)));
         const int c0 = seg * a.S - (a.K - 1);
@@ -273,7 +275,7 @@ __device__ __forceinline__ bool run_item(Block<L> &B, const OlsArgs &a, const CU
     }
 
     for (int z = z0; z < z1; ++z) {
-        if (ONE && z + 1 == z1) launch_dependents();   // (see launch_lc)
+        if (ONE && last && z + 1 == z1) launch_dependents();   // (see launch_lc)
         // output row and shift of this template (identity unless the plan groups templates)
         int row = z;
         int64_t shift = 0;
@@ -486,6 +488,42 @@ __global__ void __launch_bounds__(L / 16, MINB)
     release_block<L, 1>(B);
 }
 
+// Equal shares: block b of gridDim.x takes units [b T / gridDim.x, (b + 1) T / gridDim.x) of the
+// launch's T = nseg M (segment, template) units, segment-major, as one item per segment it
+// touches; the first item's loads start with the block, a following item's segment is fetched
+// behind the last template of the one before.  Bits as from ols_fp32_kernel.
+template <int L, int MINB>
+__global__ void __launch_bounds__(L / 16, MINB)
+    ols_fp32_shares(const __grid_constant__ CUtensorMap tmap, const OlsArgs a, int nseg)
+{
+    extern __shared__ unsigned char smem_raw[];
+    Block<L> B(smem_raw);
+    const int64_t units = (int64_t)nseg * a.M, u0 = units * blockIdx.x / gridDim.x;
+    int seg = a.seg_begin + (int)(u0 / a.M), z = (int)(u0 % a.M);
+    int64_t left = units * (blockIdx.x + 1) / gridDim.x - u0;   // >= 1: no more blocks than units
+    auto end = [&]() { return (int)min((int64_t)a.M, z + left); };
+    init_block<L, 1>(B, a, [&]() { issue_loads(B, a, &tmap, seg, z, end()); });
+    wait_prerequisites();   // before any output is written
+    bool issued = true, prefetched = false;
+    for (;;) {
+        const int z1 = end();
+        left -= z1 - z;
+        auto next = [&](const CUtensorMap **m, int *c0) -> bool {
+            *m = &tmap;
+            *c0 = (seg + 1) * a.S - (a.K - 1);
+            return left > 0;
+        };
+        if (!run_item<L, false, decltype(next), true>(B, a, &tmap, seg, z, z1, a.n, a.out, prefetched, next, issued, left == 0)) break;
+        if (left == 0) break;
+        __syncthreads();
+        ++seg;
+        z = 0;
+        issued = false;
+        prefetched = hbuf<L>() == 1;
+    }
+    release_block<L, 1>(B);
+}
+
 // Array of a batch item: the last array whose first item is <= item.
 __device__ __forceinline__ int batch_array_of(const BatchTable &tab, int64_t item)
 {
@@ -558,9 +596,11 @@ template <int L, bool CAND>
 static cudaError_t launch_lc(const CUtensorMap *tmap, const OlsArgs &a, int nseg, cudaStream_t s)
 {
     auto kern = ols_fp32_kernel<L, minb<L>(), CAND>;
+    auto shares = ols_fp32_shares<L, minb<L>()>;
     constexpr size_t smem = Smem<L>::total + (CAND ? kCandSmem : 0);
-    static bool done[64] = {};
-    cudaError_t e = set_smem_attr<L>((const void *)kern, done, smem);
+    const bool eq = !CAND && a.blocks > 0;
+    static bool done[2][64] = {};
+    cudaError_t e = set_smem_attr<L>(eq ? (const void *)shares : (const void *)kern, done[eq], smem);
     if (e != cudaSuccess) return e;
     // Programmatic dependent launch: blocks start, allocate their tensor memory and read their
     // twiddles while the launch before drains, and wait for its end before they read the input or
@@ -574,13 +614,13 @@ static cudaError_t launch_lc(const CUtensorMap *tmap, const OlsArgs &a, int nseg
     attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr.val.programmaticStreamSerializationAllowed = 1;
     cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3(nseg, (a.M + a.G - 1) / a.G);
+    cfg.gridDim = eq ? dim3(a.blocks) : dim3(nseg, (a.M + a.G - 1) / a.G);
     cfg.blockDim = dim3(L / 16);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = s;
     cfg.attrs = &attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kern, *tmap, a);
+    return eq ? cudaLaunchKernelEx(&cfg, shares, *tmap, a, nseg) : cudaLaunchKernelEx(&cfg, kern, *tmap, a);
 }
 
 template <int L>
