@@ -210,7 +210,8 @@ __device__ __forceinline__ bool run_item(Block<L> &B, const OlsArgs &a, const CU
                                          int z1, int64_t n, float *out, bool prefetched = false, Next next = Next(),
                                          bool issued = ONE, bool last = true)
 {
-    constexpr bool VMASK = ONE && !CAND;
+    constexpr bool VMASK = ONE;
+    static_assert(!(ONE && CAND), "the threshold kernel issues its own loads");
     using Gm = Geo<L>;
     constexpr int NT = Gm::NT, Q = Gm::Q, R = Gm::R, GB = Gm::GB, GC = Gm::GC, LD2 = Gm::LD2;
     constexpr uint32_t HBYTES = (uint32_t)Smem<L>::h_bytes;
@@ -482,10 +483,18 @@ __global__ void __launch_bounds__(L / 16, MINB)
         if (threadIdx.x == 0) *B.sc = 0;
     }
     const int seg = a.seg_begin + blockIdx.x, z0 = blockIdx.y * a.G, z1 = min(z0 + a.G, a.M);
-    init_block<L, 1>(B, a, [&]() { issue_loads(B, a, &tmap, seg, z0, z1); });   // its barriers also publish *B.sc = 0
-    wait_prerequisites();   // before any output is written
-    run_item<L, CAND, NoNext, true>(B, a, &tmap, seg, z0, z1, a.n, a.out);
-    release_block<L, 1>(B);
+    if constexpr (CAND) {
+        // neither early loads nor overlapped launches: 2^22 points at T_g (with the caller's sort)
+        // 811 us, 821 .. 837 with them
+        init_block<L, 0>(B, a, []() {});   // its barriers also publish *B.sc = 0
+        run_item<L, true>(B, a, &tmap, seg, z0, z1, a.n, a.out);
+        release_block<L, 0>(B);
+    } else {
+        init_block<L, 1>(B, a, [&]() { issue_loads(B, a, &tmap, seg, z0, z1); });
+        wait_prerequisites();   // before any output is written
+        run_item<L, false, NoNext, true>(B, a, &tmap, seg, z0, z1, a.n, a.out);
+        release_block<L, 1>(B);
+    }
 }
 
 // Equal shares: block b of gridDim.x takes units [b T / gridDim.x, (b + 1) T / gridDim.x) of the
@@ -619,7 +628,7 @@ static cudaError_t launch_lc(const CUtensorMap *tmap, const OlsArgs &a, int nseg
     cfg.dynamicSmemBytes = smem;
     cfg.stream = s;
     cfg.attrs = &attr;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = CAND ? 0 : 1;   // (threshold kernel: see ols_fp32_kernel)
     return eq ? cudaLaunchKernelEx(&cfg, shares, *tmap, a, nseg) : cudaLaunchKernelEx(&cfg, kern, *tmap, a);
 }
 
