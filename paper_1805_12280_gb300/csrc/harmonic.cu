@@ -17,8 +17,8 @@
 //
 // Planes narrower than 2^31 columns take one launch that walks the plane in slope windows (below)
 // with code compiled for each number of harmonics that lie in the plane; crossings are staged
-// per warp, with no block barrier.  85 x 2^22, 8 harmonics: 326 us, 1.44 GB read from DRAM (the
-// plane once), against 597 us and 3.40 GB when rows were launched in runs of equal harmonic
+// per warp, with no block barrier.  85 x 2^22, 8 harmonics: 324 us, 1.71 GB of DRAM traffic (1.2
+// planes), against 597 us and 3.40 GB when rows were launched in runs of equal harmonic
 // count and every strided pass fetched its rows again; 32 harmonics 842 -> 508 us, one harmonic
 // 272 -> 228 us, 65536 columns 61 -> 23 us per call (15 launches -> 1).  What bounds it: load
 // latency at 16 warps per SM (issue 40 %, DRAM 58 % of the measured copy rate); three blocks per SM

@@ -518,6 +518,10 @@ __device__ __forceinline__ void tc2_body(const Src &src, const tc2::Args &a)
                     }
                     tmem_fence_after_sync();
                     const uint4 *hrow = reinterpret_cast<const uint4 *>(hb + slot * H_BYTES + k2 * H_ROW);
+                    // half2 lanes = two k1, so that neither operand needs a lane broadcast (one k1 per
+                    // half2, re and im in its lanes: 2^22 points 430.4 us, a batch of 24 2973; so:
+                    // 425.8, 2930).  One role of the pipeline among several: all of its arithmetic
+                    // halved would give 2 % more.
                     uint32_t y[32];
 #pragma unroll
                     for (int c = 0; c < 8; ++c) {
