@@ -21,7 +21,7 @@
 // planes), against 597 us and 3.40 GB when rows were launched in runs of equal harmonic
 // count and every strided pass fetched its rows again; 32 harmonics 842 -> 508 us, one harmonic
 // 272 -> 228 us, 65536 columns 61 -> 23 us per call (15 launches -> 1).  What bounds it: load
-// latency at 16 warps per SM (issue 40 %, DRAM 58 % of the measured copy rate); three blocks per SM
+// latency at 16 warps per SM (issue 40 %, DRAM 78 % of the measured copy rate); three blocks per SM
 // (fewer loads in flight per thread) are 6 % slower.
 // Wider rows (and more than 4097 of them) take the general kernel with 64-bit indexing.
 #include <cuda_runtime.h>
