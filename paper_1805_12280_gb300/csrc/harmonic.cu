@@ -136,11 +136,23 @@ __global__ void __launch_bounds__(kHsThreads) harmonic_kernel(const float *__res
 // and a warp reserves its staged records with one atomic once 32 or more are waiting.
 constexpr int kWarpStage = 64, kWarpFlush = 32;
 
-__device__ __forceinline__ void warp_flush(fdas_harmonic_candidate *stage, unsigned *n_staged, int lane,
+// The warp's count of staged records, the same for every lane: read between two barriers, after all
+// of this tile's appends and before any of the next one's.  (Without the second one a lane could
+// append again while another has yet to read, and the two would part over the flush.)
+__device__ __forceinline__ unsigned warp_staged(const unsigned *n_staged)
+{
+    __syncwarp();
+    const unsigned ns = *n_staged;
+    __syncwarp();
+    return ns;
+}
+
+// All lanes, with the same `staged` from warp_staged.
+__device__ __forceinline__ void warp_flush(fdas_harmonic_candidate *stage, unsigned *n_staged, unsigned staged, int lane,
                                            fdas_harmonic_candidate *__restrict__ out, int64_t max_cand,
                                            unsigned long long *__restrict__ count)
 {
-    const unsigned ns = min(*n_staged, (unsigned)kWarpStage);
+    const unsigned ns = min(staged, (unsigned)kWarpStage);
     unsigned long long base = 0;
     if (lane == 0 && ns) base = atomicAdd(count, (unsigned long long)ns);
     base = __shfl_sync(0xffffffffu, base, 0);
@@ -266,11 +278,11 @@ __global__ void __launch_bounds__(kHsThreads, 2) harmonic_kernel_rows(const floa
     for (int64_t tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
         const int y = (int)(tile / tiles_per_row), first = 1 + (int)(tile - (int64_t)y * tiles_per_row) * kHsThreads * Q;
         hs_tile<1, Q>(P, c, n, bin0, y - c, first, lim.r_lim[1], thr, lim, stage[warp], &n_staged[warp], out, max_cand, count);
-        __syncwarp();
-        if (n_staged[warp] >= (unsigned)kWarpFlush) warp_flush(stage[warp], &n_staged[warp], lane, out, max_cand, count);
+        const unsigned ns = warp_staged(&n_staged[warp]);
+        if (ns >= (unsigned)kWarpFlush) warp_flush(stage[warp], &n_staged[warp], ns, lane, out, max_cand, count);
     }
-    __syncwarp();
-    if (n_staged[warp]) warp_flush(stage[warp], &n_staged[warp], lane, out, max_cand, count);
+    const unsigned ns = warp_staged(&n_staged[warp]);
+    if (ns) warp_flush(stage[warp], &n_staged[warp], ns, lane, out, max_cand, count);
 }
 
 template <int H>
@@ -346,11 +358,11 @@ __global__ void __launch_bounds__(kHsThreads, 2) harmonic_kernel_slope(const flo
             FDAS_HS_CASE(32)
         }
 #undef FDAS_HS_CASE
-        __syncwarp();
-        if (n_staged[warp] >= (unsigned)kWarpFlush) warp_flush(stage[warp], &n_staged[warp], lane, out, max_cand, count);
+        const unsigned ns = warp_staged(&n_staged[warp]);
+        if (ns >= (unsigned)kWarpFlush) warp_flush(stage[warp], &n_staged[warp], ns, lane, out, max_cand, count);
     }
-    __syncwarp();
-    if (n_staged[warp]) warp_flush(stage[warp], &n_staged[warp], lane, out, max_cand, count);
+    const unsigned ns = warp_staged(&n_staged[warp]);
+    if (ns) warp_flush(stage[warp], &n_staged[warp], ns, lane, out, max_cand, count);
 }
 
 // Blocks of `fn` that are resident at once (at most `tiles`); asked for once per kernel and device.
