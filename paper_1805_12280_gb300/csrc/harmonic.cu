@@ -132,34 +132,25 @@ __global__ void __launch_bounds__(kHsThreads) harmonic_kernel(const float *__res
 }
 
 // Planes of fewer than 2^31 columns: fundamentals, bins and the in-row offsets are 32-bit.
-// Crossings are staged per warp (no block barrier: each warp runs its tiles at its own pace)
-// and a warp reserves its staged records with one atomic once 32 or more are waiting.
-constexpr int kWarpStage = 64, kWarpFlush = 32;
+// Crossings are staged per warp (no block barrier: each warp runs its tiles at its own pace).  Their
+// slots come from a ballot and the count of staged records is in a register of every lane, the same
+// in all of them; a warp reserves its staged records with one atomic when the next ones may not fit.
+// 85 x 2^22, thresholds that 1 / 5 / 20 % of the sums cross: one harmonic 243 / 372 / 1113 us, eight
+// 399 / 607 / 1638, against 243 / 1253 / 3124 and 398 / 1752 / 4659 with slots from a shared counter
+// and a global reservation of its own for each record past 64 of a tile.
+constexpr int kWarpStage = 64;
 
-// The warp's count of staged records, the same for every lane: read between two barriers, after all
-// of this tile's appends and before any of the next one's.  (Without the second one a lane could
-// append again while another has yet to read, and the two would part over the flush.)
-__device__ __forceinline__ unsigned warp_staged(const unsigned *n_staged)
-{
-    __syncwarp();
-    const unsigned ns = *n_staged;
-    __syncwarp();
-    return ns;
-}
-
-// All lanes, with the same `staged` from warp_staged.
-__device__ __forceinline__ void warp_flush(fdas_harmonic_candidate *stage, unsigned *n_staged, unsigned staged, int lane,
+// All lanes, after their last stores to `stage`; it is free again on return.
+__device__ __forceinline__ void warp_flush(const fdas_harmonic_candidate *stage, unsigned staged, int lane,
                                            fdas_harmonic_candidate *__restrict__ out, int64_t max_cand,
                                            unsigned long long *__restrict__ count)
 {
-    const unsigned ns = min(staged, (unsigned)kWarpStage);
     unsigned long long base = 0;
-    if (lane == 0 && ns) base = atomicAdd(count, (unsigned long long)ns);
+    if (lane == 0) base = atomicAdd(count, (unsigned long long)staged);
     base = __shfl_sync(0xffffffffu, base, 0);
-    for (unsigned i = lane; i < ns; i += 32)
-        if ((long long)(base + i) < max_cand) out[base + i] = stage[i];
     __syncwarp();
-    if (lane == 0) *n_staged = 0;
+    for (unsigned i = lane; i < staged; i += 32)
+        if ((long long)(base + i) < max_cand) out[base + i] = stage[i];
     __syncwarp();
 }
 
@@ -184,12 +175,13 @@ __host__ __device__ constexpr int hs_levels(int kz) { return kz < 2 ? 1 : 1 + hs
 
 // One tile of 256 Q fundamentals r0 + threadIdx.x + 256 q <= rend of row z, compiled for
 // exactly the KZ harmonics that lie in the plane's drift range.  The straight-line part only
-// marks crossings in a mask; the few marked ones are appended by one short loop, so that the
-// bodies of all KZ stay small (with an append per sum the kernel was bound by instruction fetch).
+// marks crossings in a mask; the marked ones are appended by one short loop, a record per lane and
+// round, so that the bodies of all KZ stay small (with an append per sum the kernel was bound by
+// instruction fetch).  `staged`: records in the warp's stage, before and after.
 template <int KZ, int Q = hs_q(KZ)>
 __device__ __forceinline__ void hs_tile(const float *__restrict__ P, int c, int n, int bin0, int z, int r0, int rend,
                                         const HsThresholds &thr, const HsLimits &lim, fdas_harmonic_candidate *stage,
-                                        unsigned *n_staged, fdas_harmonic_candidate *__restrict__ out, int64_t max_cand,
+                                        unsigned &staged, fdas_harmonic_candidate *__restrict__ out, int64_t max_cand,
                                         unsigned long long *__restrict__ count)
 {
     constexpr int LV = hs_levels(KZ);
@@ -231,32 +223,33 @@ __device__ __forceinline__ void hs_tile(const float *__restrict__ P, int c, int 
         }
     }
     mask &= valid;
-    while (mask) {
-        const int b = (BITS == 6 ? __ffsll((long long)mask) : __ffs((int)mask)) - 1, j = b / Q;
-        mask &= mask - 1;
-        float t[1 << BITS];   // the sums by bit, then a tree of selects on the bits of b
-#pragma unroll
-        for (int i = 0; i < (1 << BITS); ++i) t[i] = i < Q * LV ? v[i % Q][(1 << (i / Q < LV ? i / Q : 0)) - 1] : 0.f;
-#pragma unroll
-        for (int bit = 0; bit < BITS; ++bit) {
-            const bool up = (b >> bit) & 1;
-#pragma unroll
-            for (int i = 0; i < ((1 << BITS) >> (bit + 1)); ++i) t[i] = up ? t[2 * i + 1] : t[2 * i];
+    const int lane = threadIdx.x & 31;
+    for (unsigned act; (act = __ballot_sync(0xffffffffu, mask != 0)) != 0;) {
+        if (staged + __popc(act) > (unsigned)kWarpStage) {
+            warp_flush(stage, staged, lane, out, max_cand, count);
+            staged = 0;
         }
-        const float power = t[0];
-        fdas_harmonic_candidate rec;
-        rec.tpl = c + z;
-        rec.power = power;
-        rec.bin = bin0 + rt + (b - Q * j) * kHsThreads;
-        rec.nharm = 1 << j;
-        rec.reserved = 0;
-        const unsigned slot = atomicAdd(n_staged, 1u);
-        if (slot < (unsigned)kWarpStage) {
-            stage[slot] = rec;
-        } else {   // staging full: reserve this record on its own
-            const unsigned long long at = atomicAdd(count, 1ull);
-            if ((long long)at < max_cand) out[at] = rec;
+        if (mask) {
+            const int b = (BITS == 6 ? __ffsll((long long)mask) : __ffs((int)mask)) - 1, j = b / Q;
+            mask &= mask - 1;
+            float t[1 << BITS];   // the sums by bit, then a tree of selects on the bits of b
+#pragma unroll
+            for (int i = 0; i < (1 << BITS); ++i) t[i] = i < Q * LV ? v[i % Q][(1 << (i / Q < LV ? i / Q : 0)) - 1] : 0.f;
+#pragma unroll
+            for (int bit = 0; bit < BITS; ++bit) {
+                const bool up = (b >> bit) & 1;
+#pragma unroll
+                for (int i = 0; i < ((1 << BITS) >> (bit + 1)); ++i) t[i] = up ? t[2 * i + 1] : t[2 * i];
+            }
+            fdas_harmonic_candidate rec;
+            rec.tpl = c + z;
+            rec.power = t[0];
+            rec.bin = bin0 + rt + (b - Q * j) * kHsThreads;
+            rec.nharm = 1 << j;
+            rec.reserved = 0;
+            stage[staged + __popc(act & ((1u << lane) - 1u))] = rec;
         }
+        staged += __popc(act);
     }
 }
 
@@ -270,19 +263,14 @@ __global__ void __launch_bounds__(kHsThreads, 2) harmonic_kernel_rows(const floa
                                                                       unsigned long long *__restrict__ count)
 {
     __shared__ fdas_harmonic_candidate stage[kHsThreads / 32][kWarpStage];
-    __shared__ unsigned n_staged[kHsThreads / 32];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    if (lane == 0) n_staged[warp] = 0;
-    __syncwarp();
+    unsigned staged = 0;
     const int64_t tiles = (int64_t)(2 * c + 1) * tiles_per_row;
     for (int64_t tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
         const int y = (int)(tile / tiles_per_row), first = 1 + (int)(tile - (int64_t)y * tiles_per_row) * kHsThreads * Q;
-        hs_tile<1, Q>(P, c, n, bin0, y - c, first, lim.r_lim[1], thr, lim, stage[warp], &n_staged[warp], out, max_cand, count);
-        const unsigned ns = warp_staged(&n_staged[warp]);
-        if (ns >= (unsigned)kWarpFlush) warp_flush(stage[warp], &n_staged[warp], ns, lane, out, max_cand, count);
+        hs_tile<1, Q>(P, c, n, bin0, y - c, first, lim.r_lim[1], thr, lim, stage[warp], staged, out, max_cand, count);
     }
-    const unsigned ns = warp_staged(&n_staged[warp]);
-    if (ns) warp_flush(stage[warp], &n_staged[warp], ns, lane, out, max_cand, count);
+    if (staged) warp_flush(stage[warp], staged, lane, out, max_cand, count);
 }
 
 template <int H>
@@ -293,7 +281,6 @@ __global__ void __launch_bounds__(kHsThreads, 2) harmonic_kernel_slope(const flo
                                                                        unsigned long long *__restrict__ count)
 {
     __shared__ fdas_harmonic_candidate stage[kHsThreads / 32][kWarpStage];
-    __shared__ unsigned n_staged[kHsThreads / 32];
     extern __shared__ int4 ent[];   // entry (window, |z| = c .. 1): its end in tiles, first and last
                                     // fundamental, |z| << 14 | fundamentals per thread << 6 | harmonics
     __shared__ int part[kHsThreads / 32];
@@ -318,7 +305,6 @@ __global__ void __launch_bounds__(kHsThreads, 2) harmonic_kernel_slope(const flo
             if (lane >= o) incl += v;
         }
         if (lane == 31) part[warp] = incl;
-        if (lane == 0) n_staged[warp] = 0;
         __syncthreads();
         int before = incl - sum;
         for (int i = 0; i < warp; ++i) before += part[i];
@@ -328,6 +314,7 @@ __global__ void __launch_bounds__(kHsThreads, 2) harmonic_kernel_slope(const flo
     constexpr int TILE0 = kHsThreads * hs_q(H);
     const int tiles0 = (rmax + TILE0 - 1) / TILE0;   // of the z = 0 row
     const int tiles = tiles0 + (entries ? ent[entries - 1].x : 0);
+    unsigned staged = 0;
     int e = 0, begin = 0;   // the entry of this block's tile, and its first tile
     for (int tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
         int z = 0, kz = H, first = 1 + tile * TILE0, last = rmax;
@@ -347,7 +334,7 @@ __global__ void __launch_bounds__(kHsThreads, 2) harmonic_kernel_slope(const flo
 #define FDAS_HS_CASE(K)                                                                                                   \
     case K:                                                                                                                \
         if constexpr (K <= H)                                                                                              \
-            hs_tile<K>(P, c, n, bin0, z, first, last, thr, lim, stage[warp], &n_staged[warp], out, max_cand, count);       \
+            hs_tile<K>(P, c, n, bin0, z, first, last, thr, lim, stage[warp], staged, out, max_cand, count);                \
         break;
         switch (kz) {
             FDAS_HS_CASE(1) FDAS_HS_CASE(2) FDAS_HS_CASE(3) FDAS_HS_CASE(4) FDAS_HS_CASE(5) FDAS_HS_CASE(6) FDAS_HS_CASE(7)
@@ -358,11 +345,8 @@ __global__ void __launch_bounds__(kHsThreads, 2) harmonic_kernel_slope(const flo
             FDAS_HS_CASE(32)
         }
 #undef FDAS_HS_CASE
-        const unsigned ns = warp_staged(&n_staged[warp]);
-        if (ns >= (unsigned)kWarpFlush) warp_flush(stage[warp], &n_staged[warp], ns, lane, out, max_cand, count);
     }
-    const unsigned ns = warp_staged(&n_staged[warp]);
-    if (ns) warp_flush(stage[warp], &n_staged[warp], ns, lane, out, max_cand, count);
+    if (staged) warp_flush(stage[warp], staged, lane, out, max_cand, count);
 }
 
 // Blocks of `fn` that are resident at once (at most `tiles`); asked for once per kernel and device.
