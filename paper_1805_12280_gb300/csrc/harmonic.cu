@@ -317,8 +317,10 @@ __global__ void __launch_bounds__(kHsThreads, 2) harmonic_kernel_slope(const flo
     unsigned staged = 0;
     int e = 0, begin = 0;   // the entry of this block's tile, and its first tile
     for (int tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
-        int z = 0, kz = H, first = 1 + tile * TILE0, last = rmax;
-        if (tile >= tiles0) {
+        int z = 0, kz = H, first, last = rmax;
+        if (tile < tiles0) {
+            first = 1 + tile * TILE0;
+        } else {
             const int t = tile - tiles0;
             int4 en = ent[e];
             while (t >= en.x) {
