@@ -23,7 +23,8 @@
 // 272 -> 228 us, 65536 columns 61 -> 23 us per call (15 launches -> 1).  What bounds it: load
 // latency at 16 warps per SM (issue 40 %, DRAM 78 % of the measured copy rate); three blocks per SM
 // (fewer loads in flight per thread) are 6 % slower.
-// Wider rows (and more than 4097 of them) take the general kernel with 64-bit indexing.
+// Planes of more than 2049 rows, whose table has no room for two windows, go by runs of rows with the
+// same number of harmonics in the same launch.  Wider rows take the general kernel with 64-bit indexing.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -164,7 +165,7 @@ __device__ __forceinline__ void warp_flush(const fdas_harmonic_candidate *stage,
 constexpr int kHsMaxWin = 128, kHsMaxEntries = 2048;   // windows; (window, |z|) entries of one launch
 constexpr int64_t kHsWindowBytes = 64ll << 20;
 struct HsWindows {
-    int count;
+    int count;   // 0: the plane as a whole, by runs of rows with the same number of harmonics
     int slope[kHsMaxWin + 1];
 };
 
@@ -273,7 +274,8 @@ __global__ void __launch_bounds__(kHsThreads, 2) harmonic_kernel_rows(const floa
     if (staged) warp_flush(stage[warp], staged, lane, out, max_cand, count);
 }
 
-template <int H>
+// RUNS: not by windows but by runs of rows with the same number of harmonics (win.count = 0).
+template <int H, bool RUNS>
 __global__ void __launch_bounds__(kHsThreads, 2) harmonic_kernel_slope(const float *__restrict__ P, int c, int n, int bin0,
                                                                        HsThresholds thr, HsLimits lim, HsWindows win,
                                                                        fdas_harmonic_candidate *__restrict__ out,
@@ -282,14 +284,22 @@ __global__ void __launch_bounds__(kHsThreads, 2) harmonic_kernel_slope(const flo
 {
     __shared__ fdas_harmonic_candidate stage[kHsThreads / 32][kWarpStage];
     extern __shared__ int4 ent[];   // entry (window, |z| = c .. 1): its end in tiles, first and last
-                                    // fundamental, |z| << 14 | fundamentals per thread << 6 | harmonics
+                                    // fundamental, |z| << 14 | fundamentals per thread << 6 | harmonics;
+                                    // entry of a run of rows: its end in tiles, tiles per row, largest
+                                    // |z|, fundamentals per thread << 6 | harmonics
     __shared__ int part[kHsThreads / 32];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int rmax = lim.r_lim[1], entries = win.count * c;
+    const int rmax = lim.r_lim[1], entries = RUNS ? min(min(H, c), rmax) : win.count * c;
     {   // tile counts: each thread sums a run of entries, then a block scan
         const int per = (entries + kHsThreads - 1) / kHsThreads, e0 = min(tid * per, entries), e1 = min(e0 + per, entries);
         int sum = 0;
         for (int e = e0; e < e1; ++e) {
+            if constexpr (RUNS) {   // rows c / (e + 2) < |z| <= c / (e + 1); the last run: all that are left
+                const int kz = e + 1, hi = c / kz, tile = kHsThreads * hs_q(kz), per_row = (rmax + tile - 1) / tile;
+                sum += 2 * (hi - (kz == entries ? 0 : c / (kz + 1))) * per_row;
+                ent[e] = make_int4(sum, per_row, hi, (hs_q(kz) << 6) | kz);
+                continue;
+            }
             const int w = e / c, a = c - (e - w * c);
             const int64_t lo = (int64_t)a * win.slope[w], hi = (int64_t)a * win.slope[w + 1];
             const int first = (int)(lo < rmax ? lo : rmax) + 1, last = (int)(hi < rmax ? hi : rmax);
@@ -329,9 +339,15 @@ __global__ void __launch_bounds__(kHsThreads, 2) harmonic_kernel_slope(const flo
             }
             const int local = t - begin, half = (en.x - begin) >> 1;
             kz = en.w & 63;
-            z = local < half ? en.w >> 14 : -(en.w >> 14);
-            first = en.y + (local < half ? local : local - half) * kHsThreads * ((en.w >> 6) & 255);
-            last = en.z;
+            if constexpr (RUNS) {
+                const int at = local < half ? local : local - half, row = at / en.y;
+                z = local < half ? en.z - row : row - en.z;
+                first = 1 + (at - row * en.y) * kHsThreads * (en.w >> 6);
+            } else {
+                z = local < half ? en.w >> 14 : -(en.w >> 14);
+                first = en.y + (local < half ? local : local - half) * kHsThreads * ((en.w >> 6) & 255);
+                last = en.z;
+            }
         }
 #define FDAS_HS_CASE(K)                                                                                                   \
     case K:                                                                                                                \
@@ -375,8 +391,11 @@ cudaError_t launch_hs(int H, const float *P, int m, int64_t n, int64_t bin0, con
     const int c = (m - 1) / 2;
     cudaError_t e;
     unsigned grid = 0;
-    // 32-bit fundamentals and bins, with room for the last tile's overhang past rmax
-    if (n <= (((int64_t)1 << 31) - ((int64_t)1 << 16)) && c <= kHsMaxEntries) {
+    // at most one tile per 256 fundamentals of a row and one more for each end of a window
+    const int64_t most_tiles = (int64_t)m * (rmax / kHsThreads + 1) + 2 * (int64_t)kHsMaxEntries;
+    // 32-bit fundamentals and bins, with room for the last tile's overhang past rmax, and tiles
+    const int64_t limit = ((int64_t)1 << 31) - ((int64_t)1 << 16);
+    if (n <= limit && (H == 1 || most_tiles <= limit)) {
         HsLimits lim{};
         for (int k = 1; k <= 32; ++k) lim.r_lim[k] = (int)(rmax / k);
         if (H == 1) {
@@ -393,35 +412,40 @@ cudaError_t launch_hs(int H, const float *P, int m, int64_t n, int64_t bin0, con
             }
             return cudaGetLastError();
         }
+        // windows of about kHsWindowBytes of the plane: rows |z| <= rmax / S reach slope S.  Where the
+        // table has no room for two, the rows go in runs (4099 x 65536, default thresholds, eight / 32
+        // harmonics: 383 / 575 us, 1763 / 5503 by the 64-bit kernel)
         HsWindows win{};
-        // windows of about kHsWindowBytes of the plane: rows |z| <= rmax / S reach slope S
-        int64_t S = 0, bytes = kHsWindowBytes;
-        const int most = c > 0 ? std::min(kHsMaxWin, kHsMaxEntries / c) : 1;
+        const int most = c > 0 ? std::min(kHsMaxWin, kHsMaxEntries / c) : 0;
         const int64_t plane = (int64_t)m * n * 4;
-        if (plane / most > bytes) bytes = plane / most;
-        while (S < rmax && c > 0) {
-            const int64_t a = std::min<int64_t>(c, S > 0 ? rmax / S : c);
-            S += std::max<int64_t>(1, bytes / (4 * a * (a + 1)));
-            if (win.count == most - 1 || S > rmax) S = rmax;
-            win.slope[++win.count] = (int)S;
+        if (most > 1) {
+            const int64_t bytes = std::max(kHsWindowBytes, plane / most);
+            for (int64_t S = 0; S < rmax;) {
+                const int64_t a = std::min<int64_t>(c, S > 0 ? rmax / S : c);
+                S += std::max<int64_t>(1, bytes / (4 * a * (a + 1)));
+                if (win.count == most - 1 || S > rmax) S = rmax;
+                win.slope[++win.count] = (int)S;
+            }
         }
+        const size_t table = sizeof(int4) * (win.count ? (size_t)win.count * c : 32);
         using Kernel = void (*)(const float *, int, int, int, HsThresholds, HsLimits, HsWindows, fdas_harmonic_candidate *,
                                 int64_t, unsigned long long *);
-        Kernel fn;
-        switch (H) {
-        case 2: fn = harmonic_kernel_slope<2>; break;
-        case 4: fn = harmonic_kernel_slope<4>; break;
-        case 8: fn = harmonic_kernel_slope<8>; break;
-        case 16: fn = harmonic_kernel_slope<16>; break;
-        default: fn = harmonic_kernel_slope<32>; break;
-        }
-        // at most one tile per block: both signs of every row, its ragged ends, and the z = 0 row
-        const int64_t tiles = (int64_t)m * (rmax / kHsThreads + 1) + 2 * (int64_t)c * win.count;
+        auto kernel = [&](auto runs) -> Kernel {
+            switch (H) {
+            case 2: return harmonic_kernel_slope<2, runs()>;
+            case 4: return harmonic_kernel_slope<4, runs()>;
+            case 8: return harmonic_kernel_slope<8, runs()>;
+            case 16: return harmonic_kernel_slope<16, runs()>;
+            default: return harmonic_kernel_slope<32, runs()>;
+            }
+        };
+        const bool runs = win.count == 0;
+        const Kernel fn = runs ? kernel(std::true_type()) : kernel(std::false_type());
         // (the occupancy of the largest table, so that one number serves every call)
-        static std::atomic<int> known[6][64];
+        static std::atomic<int> known[2][6][64];
         const int level = 31 - __builtin_clz((unsigned)H);
-        if ((e = resident_grid((const void *)fn, tiles, sizeof(int4) * kHsMaxEntries, known[level], &grid)) != cudaSuccess) return e;
-        fn<<<grid, kHsThreads, sizeof(int4) * (size_t)(win.count * c), s>>>(P, c, (int)n, (int)bin0, thr, lim, win, out, max_cand, count);
+        if ((e = resident_grid((const void *)fn, most_tiles, sizeof(int4) * kHsMaxEntries, known[runs][level], &grid)) != cudaSuccess) return e;
+        fn<<<grid, kHsThreads, table, s>>>(P, c, (int)n, (int)bin0, thr, lim, win, out, max_cand, count);
         return cudaGetLastError();
     }
     const void *fn = nullptr;

@@ -51,3 +51,22 @@ def test_crossing_sets(fd, oracle_mod, m, n, bin0, H):
     value = ref["value"][at_want]
     h = levels[ref["level"][at_want]]
     assert np.all(np.abs(got["power"][at_have].astype(np.float64) - value) <= (h - 1) * U / (1 - (h - 1) * U) * value)
+
+
+@pytest.mark.parametrize("m,n,bin0,H", [(4099, 1_025, 0, 32), (4097, 2_000, 3, 8), (20_001, 41, 2, 8),   # rows of |z| > c / H in runs
+                                        (8193, 6, 0, 32),             # fewer columns than harmonics
+                                        (2_051, 700, 0, 16), (2_049, 700, 0, 16), (85, 13_000, 210, 2), (3, 3, 0, 2)])
+def test_planes_walked_by_rows(fd, oracle_mod, m, n, bin0, H):
+    # more rows than the window table holds twice, and planes beside that limit: every defined sum
+    P = synth.noise_plane(m, n, seed=n + H)
+    S = oracle_mod.harmonic_sums(P, bin0, H)
+    levels = np.array(fd.harmonic_levels(H))
+    total = int((~np.isnan(S)).sum())
+    buf, count = fd.harmonic_sum(torch.from_numpy(P).cuda(), bin0, H, [-1.0] * levels.size, max_cand=total + 64)
+    assert int(count.item()) == total
+    got = fd.harmonic_to_numpy(buf, count)
+    j = np.log2(got["nharm"]).astype(np.int64)
+    assert np.unique((j * m + got["tpl"]) * n + got["bin"]).size == total
+    ref = S[j, got["tpl"], got["bin"]]
+    h = levels[j]
+    assert np.all(np.abs(got["power"].astype(np.float64) - ref) <= (h - 1) * U / (1 - (h - 1) * U) * ref)
