@@ -23,7 +23,7 @@
 // 272 -> 228 us, 65536 columns 61 -> 23 us per call (15 launches -> 1).  What bounds it: load
 // latency at 16 warps per SM (issue 40 %, DRAM 78 % of the measured copy rate); three blocks per SM
 // (fewer loads in flight per thread) are 6 % slower.
-// Planes of more than 2049 rows, whose table has no room for two windows, go by runs of rows with the
+// Planes of more than 513 rows, whose table has little room for windows, go by runs of rows with the
 // same number of harmonics in the same launch.  Wider rows take the general kernel with 64-bit indexing.
 #include <cuda_runtime.h>
 
@@ -325,17 +325,23 @@ __global__ void __launch_bounds__(kHsThreads, 2) harmonic_kernel_slope(const flo
     const int tiles0 = (rmax + TILE0 - 1) / TILE0;   // of the z = 0 row
     const int tiles = tiles0 + (entries ? ent[entries - 1].x : 0);
     unsigned staged = 0;
-    int e = 0, begin = 0;   // the entry of this block's tile, and its first tile
+    // The entry of this block's tile, and its first tile.  A few entries are passed one at a time (most
+    // steps of a large plane; the vote at once costs 257 x 1.4e6, 32 harmonics 528 us against 501), many
+    // 32 at a time: a table of 750 entries costs a small plane 10 us otherwise (513 x 8000: 27 us against 17).
+    int e = 0, begin = 0;
+    int4 en = entries ? ent[0] : int4{};
     for (int tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
         int z = 0, kz = H, first, last = rmax;
         if (tile < tiles0) {
             first = 1 + tile * TILE0;
         } else {
             const int t = tile - tiles0;
-            int4 en = ent[e];
-            while (t >= en.x) {
-                begin = en.x;
-                en = ent[++e];
+            for (int i = 0; i < 8 && t >= en.x; ++i) begin = en.x, en = ent[++e];
+            if (t >= en.x) {   // the last entry's end is past t
+                int passed;
+                do e += passed = __popc(__ballot_sync(0xffffffffu, ent[min(e + lane, entries - 1)].x <= t));
+                while (passed == 32);
+                begin = ent[e - 1].x, en = ent[e];
             }
             const int local = t - begin, half = (en.x - begin) >> 1;
             kz = en.w & 63;
@@ -413,12 +419,14 @@ cudaError_t launch_hs(int H, const float *P, int m, int64_t n, int64_t bin0, con
             return cudaGetLastError();
         }
         // windows of about kHsWindowBytes of the plane: rows |z| <= rmax / S reach slope S.  Where the
-        // table has no room for two, the rows go in runs (4099 x 65536, default thresholds, eight / 32
-        // harmonics: 383 / 575 us, 1763 / 5503 by the 64-bit kernel)
+        // table has no room for eight (more than 513 rows; for four, 1025 rows, in planes well beyond
+        // L2) the rows go in runs: 1025 rows of 90 MB with two / eight / 32 harmonics 21 / 31 / 58 us, in
+        // four windows 32 / 39 / 48, 1400 MB 303 / 481 / 732 against 303 / 480 / 700; 2001 rows of 90 MB
+        // 22 / 33 / 65, in two windows 35 / 45 / 63, 1400 MB 308 / 490 / 760 against 328 / 537 / 917
         HsWindows win{};
         const int most = c > 0 ? std::min(kHsMaxWin, kHsMaxEntries / c) : 0;
         const int64_t plane = (int64_t)m * n * 4;
-        if (most > 1) {
+        if (most >= 8 || (most >= 4 && plane > (256ll << 20))) {
             const int64_t bytes = std::max(kHsWindowBytes, plane / most);
             for (int64_t S = 0; S < rmax;) {
                 const int64_t a = std::min<int64_t>(c, S > 0 ? rmax / S : c);
