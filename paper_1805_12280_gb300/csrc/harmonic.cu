@@ -163,6 +163,7 @@ __device__ __forceinline__ void warp_flush(const fdas_harmonic_candidate *stage,
 // (its harmonics lie in itself) comes first.  Windows of 64 MB (8 harmonics at 2^22, sorted
 // records included: 16 MB 766, 32 MB 711, 64 MB 693, the whole plane 771 us in one version).
 constexpr int kHsMaxWin = 128, kHsMaxEntries = 2048;   // windows; (window, |z|) entries of one launch
+constexpr size_t kHsTableBytes = sizeof(int4) * (kHsMaxEntries + 32);   // with the z = 0 row's
 constexpr int64_t kHsWindowBytes = 64ll << 20;
 struct HsWindows {
     int count;   // 0: the plane as a whole, by runs of rows with the same number of harmonics
@@ -283,21 +284,29 @@ __global__ void __launch_bounds__(kHsThreads, 2) harmonic_kernel_slope(const flo
                                                                        unsigned long long *__restrict__ count)
 {
     __shared__ fdas_harmonic_candidate stage[kHsThreads / 32][kWarpStage];
-    extern __shared__ int4 ent[];   // entry (window, |z| = c .. 1): its end in tiles, first and last
-                                    // fundamental, |z| << 14 | fundamentals per thread << 6 | harmonics;
-                                    // entry of a run of rows: its end in tiles, tiles per row, largest
-                                    // |z|, fundamentals per thread << 6 | harmonics
+    // entry (z = 0, number of harmonics inside the row) and entry (window, |z| = c .. 1): its end in tiles,
+    // first and last fundamental, |z| << 14 | fundamentals per thread << 6 | harmonics; entry of a run of
+    // rows: its end in tiles, tiles per row, largest |z|, fundamentals per thread << 6 | harmonics
+    extern __shared__ int4 ent[];
     __shared__ int part[kHsThreads / 32];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int rmax = lim.r_lim[1], entries = RUNS ? min(min(H, c), rmax) : win.count * c;
+    const int rmax = lim.r_lim[1], most = min(H, rmax);   // harmonics inside a row of the plane
+    const int zeros = most, runs = min(most, c), entries = zeros + (RUNS ? runs : win.count * c);
     {   // tile counts: each thread sums a run of entries, then a block scan
         const int per = (entries + kHsThreads - 1) / kHsThreads, e0 = min(tid * per, entries), e1 = min(e0 + per, entries);
         int sum = 0;
-        for (int e = e0; e < e1; ++e) {
+        for (int i = e0; i < e1; ++i) {
+            if (i < zeros) {   // z = 0: fundamentals rmax / (i + 2) < r <= rmax / (i + 1), the rest with the most
+                const int kz = i + 1, first = kz == zeros ? 1 : lim.r_lim[kz + 1] + 1, tile = kHsThreads * hs_q(kz);
+                sum += (lim.r_lim[kz] - first + tile) / tile;
+                ent[i] = make_int4(sum, first, lim.r_lim[kz], (hs_q(kz) << 6) | kz);
+                continue;
+            }
+            const int e = i - zeros;
             if constexpr (RUNS) {   // rows c / (e + 2) < |z| <= c / (e + 1); the last run: all that are left
                 const int kz = e + 1, hi = c / kz, tile = kHsThreads * hs_q(kz), per_row = (rmax + tile - 1) / tile;
-                sum += 2 * (hi - (kz == entries ? 0 : c / (kz + 1))) * per_row;
-                ent[e] = make_int4(sum, per_row, hi, (hs_q(kz) << 6) | kz);
+                sum += 2 * (hi - (kz == runs ? 0 : c / (kz + 1))) * per_row;
+                ent[i] = make_int4(sum, per_row, hi, (hs_q(kz) << 6) | kz);
                 continue;
             }
             const int w = e / c, a = c - (e - w * c);
@@ -306,7 +315,7 @@ __global__ void __launch_bounds__(kHsThreads, 2) harmonic_kernel_slope(const flo
             // the harmonics of its first fundamental inside the plane (rows and columns)
             const int kz = max(1, min(min(H, c / a), rmax / first)), tile = kHsThreads * hs_q(kz);
             sum += 2 * ((last - first + tile) / tile);   // both signs of z
-            ent[e] = make_int4(sum, first, last, (a << 14) | (hs_q(kz) << 6) | kz);
+            ent[i] = make_int4(sum, first, last, (a << 14) | (hs_q(kz) << 6) | kz);
         }
         int incl = sum;
 #pragma unroll
@@ -318,43 +327,39 @@ __global__ void __launch_bounds__(kHsThreads, 2) harmonic_kernel_slope(const flo
         __syncthreads();
         int before = incl - sum;
         for (int i = 0; i < warp; ++i) before += part[i];
-        for (int e = e0; e < e1; ++e) ent[e].x += before;
+        for (int i = e0; i < e1; ++i) ent[i].x += before;
         __syncthreads();
     }
-    constexpr int TILE0 = kHsThreads * hs_q(H);
-    const int tiles0 = (rmax + TILE0 - 1) / TILE0;   // of the z = 0 row
-    const int tiles = tiles0 + (entries ? ent[entries - 1].x : 0);
+    const int tiles = ent[entries - 1].x;
     unsigned staged = 0;
     // The entry of this block's tile, and its first tile.  A few entries are passed one at a time (most
     // steps of a large plane; the vote at once costs 257 x 1.4e6, 32 harmonics 528 us against 501), many
     // 32 at a time: a table of 750 entries costs a small plane 10 us otherwise (513 x 8000: 27 us against 17).
     int e = 0, begin = 0;
-    int4 en = entries ? ent[0] : int4{};
+    int4 en = ent[0];
     for (int tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
-        int z = 0, kz = H, first, last = rmax;
-        if (tile < tiles0) {
-            first = 1 + tile * TILE0;
-        } else {
-            const int t = tile - tiles0;
-            for (int i = 0; i < 8 && t >= en.x; ++i) begin = en.x, en = ent[++e];
-            if (t >= en.x) {   // the last entry's end is past t
-                int passed;
-                do e += passed = __popc(__ballot_sync(0xffffffffu, ent[min(e + lane, entries - 1)].x <= t));
-                while (passed == 32);
-                begin = ent[e - 1].x, en = ent[e];
-            }
-            const int local = t - begin, half = (en.x - begin) >> 1;
-            kz = en.w & 63;
-            if constexpr (RUNS) {
-                const int at = local < half ? local : local - half, row = at / en.y;
-                z = local < half ? en.z - row : row - en.z;
-                first = 1 + (at - row * en.y) * kHsThreads * (en.w >> 6);
-            } else {
-                z = local < half ? en.w >> 14 : -(en.w >> 14);
-                first = en.y + (local < half ? local : local - half) * kHsThreads * ((en.w >> 6) & 255);
-                last = en.z;
-            }
+        for (int i = 0; i < 8 && tile >= en.x; ++i) begin = en.x, en = ent[++e];
+        if (tile >= en.x) {   // the last entry's end is past every tile
+            int passed;
+            do e += passed = __popc(__ballot_sync(0xffffffffu, ent[min(e + lane, entries - 1)].x <= tile));
+            while (passed == 32);
+            begin = ent[e - 1].x, en = ent[e];
         }
+        const int kz = en.w & 63, a = en.w >> 14, local = tile - begin;
+        int z = 0, last = rmax, at = local;   // tile of the row
+        if (!RUNS || e < zeros) {
+            const int half = (en.x - begin) >> 1;
+            last = en.z;
+            if (a) {   // both signs of z
+                z = local < half ? a : -a;
+                at = local < half ? local : local - half;
+            }
+        } else {
+            const int half = (en.x - begin) >> 1, u = local < half ? local : local - half, row = u / en.y;
+            z = local < half ? en.z - row : row - en.z;
+            at = u - row * en.y;
+        }
+        const int first = (!RUNS || e < zeros ? en.y : 1) + at * kHsThreads * ((en.w >> 6) & 255);
 #define FDAS_HS_CASE(K)                                                                                                   \
     case K:                                                                                                                \
         if constexpr (K <= H)                                                                                              \
@@ -398,7 +403,7 @@ cudaError_t launch_hs(int H, const float *P, int m, int64_t n, int64_t bin0, con
     cudaError_t e;
     unsigned grid = 0;
     // at most one tile per 256 fundamentals of a row and one more for each end of a window
-    const int64_t most_tiles = (int64_t)m * (rmax / kHsThreads + 1) + 2 * (int64_t)kHsMaxEntries;
+    const int64_t most_tiles = (int64_t)m * (rmax / kHsThreads + 1) + 2 * (int64_t)kHsMaxEntries + 32;
     // 32-bit fundamentals and bins, with room for the last tile's overhang past rmax, and tiles
     const int64_t limit = ((int64_t)1 << 31) - ((int64_t)1 << 16);
     if (n <= limit && (H == 1 || most_tiles <= limit)) {
@@ -435,7 +440,7 @@ cudaError_t launch_hs(int H, const float *P, int m, int64_t n, int64_t bin0, con
                 win.slope[++win.count] = (int)S;
             }
         }
-        const size_t table = sizeof(int4) * (win.count ? (size_t)win.count * c : 32);
+        const size_t table = sizeof(int4) * (32 + (win.count ? (size_t)win.count * c : 32));
         using Kernel = void (*)(const float *, int, int, int, HsThresholds, HsLimits, HsWindows, fdas_harmonic_candidate *,
                                 int64_t, unsigned long long *);
         auto kernel = [&](auto runs) -> Kernel {
@@ -452,7 +457,7 @@ cudaError_t launch_hs(int H, const float *P, int m, int64_t n, int64_t bin0, con
         // (the occupancy of the largest table, so that one number serves every call)
         static std::atomic<int> known[2][6][64];
         const int level = 31 - __builtin_clz((unsigned)H);
-        if ((e = resident_grid((const void *)fn, most_tiles, sizeof(int4) * kHsMaxEntries, known[runs][level], &grid)) != cudaSuccess) return e;
+        if ((e = resident_grid((const void *)fn, most_tiles, kHsTableBytes, known[runs][level], &grid)) != cudaSuccess) return e;
         fn<<<grid, kHsThreads, table, s>>>(P, c, (int)n, (int)bin0, thr, lim, win, out, max_cand, count);
         return cudaGetLastError();
     }
