@@ -173,6 +173,7 @@ struct HsWindows {
 // Fundamentals per thread of rows with kz harmonics: 48 to 64 loads in flight, and a bit per
 // (fundamental, level) in one mask (16 and 8 fundamentals for kz = 1 and 2: 609 us against 510).
 __host__ __device__ constexpr int hs_q(int kz) { return kz == 1 ? 48 : kz == 2 ? 24 : kz == 3 ? 16 : kz <= 8 ? 8 : 64 / kz; }
+constexpr int kHsTall = 2, kHsCases = 32;   // tall tiles are compiled for kz <= kHsTall, as cases above kHsCases
 __host__ __device__ constexpr int hs_levels(int kz) { return kz < 2 ? 1 : 1 + hs_levels(kz / 2); }
 
 // One tile of 256 Q fundamentals r0 + threadIdx.x + 256 q <= rend of row z, compiled for
@@ -180,7 +181,9 @@ __host__ __device__ constexpr int hs_levels(int kz) { return kz < 2 ? 1 : 1 + hs
 // marks crossings in a mask; the marked ones are appended by one short loop, a record per lane and
 // round, so that the bodies of all KZ stay small (with an append per sum the kernel was bound by
 // instruction fetch).  `staged`: records in the warp's stage, before and after.
-template <int KZ, int Q = hs_q(KZ)>
+// TALL, for rows much shorter than 256 Q: the 256 fundamentals r0 + threadIdx.x of Q rows, from z inwards,
+// `rend` of which belong to the run.
+template <int KZ, int Q = hs_q(KZ), bool TALL = false>
 __device__ __forceinline__ void hs_tile(const float *__restrict__ P, int c, int n, int bin0, int z, int r0, int rend,
                                         const HsThresholds &thr, const HsLimits &lim, fdas_harmonic_candidate *stage,
                                         unsigned &staged, fdas_harmonic_candidate *__restrict__ out, int64_t max_cand,
@@ -192,21 +195,24 @@ __device__ __forceinline__ void hs_tile(const float *__restrict__ P, int c, int 
     const int rt = r0 + (int)threadIdx.x;
     float v[Q][KZ];
     Mask valid = ~Mask(0);   // bits of the sums that are defined
-    if (r0 + kHsThreads * Q - 1 <= min(lim.r_lim[KZ], rend)) {   // every harmonic of the tile lies in the plane
+    const int64_t step = TALL ? (z < 0 ? n : -(int64_t)n) : kHsThreads;   // cells from q to q + 1
+    if (TALL ? r0 + kHsThreads - 1 <= lim.r_lim[KZ] && rend >= Q
+             : r0 + kHsThreads * Q - 1 <= min(lim.r_lim[KZ], rend)) {   // every harmonic of the tile lies in the plane
 #pragma unroll
         for (int k = 1; k <= KZ; ++k) {
             const float *base = P + ((int64_t)(c + k * z) * n + bin0 + (int64_t)k * rt);   // cell (c + k z, bin0 + k r)
 #pragma unroll
-            for (int q = 0; q < Q; ++q) v[q][k - 1] = __ldg(base + k * kHsThreads * q);
+            for (int q = 0; q < Q; ++q) v[q][k - 1] = __ldg(base + k * step * q);
         }
     } else {
         valid = 0;
 #pragma unroll
         for (int k = 1; k <= KZ; ++k) {
             const float *base = P + ((int64_t)(c + k * z) * n + bin0 + (int64_t)k * rt);
-            const int last = min(lim.r_lim[k], rend), in = last < rt ? 0 : min((last - rt) / kHsThreads + 1, Q);   // q < in
+            const int last = TALL ? lim.r_lim[k] : min(lim.r_lim[k], rend);
+            const int in = last < rt ? 0 : min(TALL ? rend : (last - rt) / kHsThreads + 1, Q);   // q < in
 #pragma unroll
-            for (int q = 0; q < Q; ++q) v[q][k - 1] = q < in ? __ldg(base + k * kHsThreads * q) : 0.f;
+            for (int q = 0; q < Q; ++q) v[q][k - 1] = q < in ? __ldg(base + k * step * q) : 0.f;
             if ((k & (k - 1)) == 0) valid |= (Mask)(in >= 64 ? ~0ull : (1ull << in) - 1) << (Q * (31 - __clz(k)));
         }
     }
@@ -244,9 +250,10 @@ __device__ __forceinline__ void hs_tile(const float *__restrict__ P, int c, int 
                 for (int i = 0; i < ((1 << BITS) >> (bit + 1)); ++i) t[i] = up ? t[2 * i + 1] : t[2 * i];
             }
             fdas_harmonic_candidate rec;
-            rec.tpl = c + z;
+            const int q = b - Q * j;
+            rec.tpl = c + (!TALL ? z : z < 0 ? z + q : z - q);
             rec.power = t[0];
-            rec.bin = bin0 + rt + (b - Q * j) * kHsThreads;
+            rec.bin = bin0 + rt + (TALL ? 0 : q * kHsThreads);
             rec.nharm = 1 << j;
             rec.reserved = 0;
             stage[staged + __popc(act & ((1u << lane) - 1u))] = rec;
@@ -275,8 +282,10 @@ __global__ void __launch_bounds__(kHsThreads, 2) harmonic_kernel_rows(const floa
     if (staged) warp_flush(stage[warp], staged, lane, out, max_cand, count);
 }
 
-// RUNS: not by windows but by runs of rows with the same number of harmonics (win.count = 0).
-template <int H, bool RUNS>
+// MODE: kWindows, or not by windows but by runs of rows with the same number of harmonics (win.count = 0),
+// kTallRuns with tall tiles (a kernel of its own: their code costs 32 harmonics in long rows 9 %).
+enum { kWindows, kRuns, kTallRuns };
+template <int H, int MODE>
 __global__ void __launch_bounds__(kHsThreads, 2) harmonic_kernel_slope(const float *__restrict__ P, int c, int n, int bin0,
                                                                        HsThresholds thr, HsLimits lim, HsWindows win,
                                                                        fdas_harmonic_candidate *__restrict__ out,
@@ -286,8 +295,10 @@ __global__ void __launch_bounds__(kHsThreads, 2) harmonic_kernel_slope(const flo
     __shared__ fdas_harmonic_candidate stage[kHsThreads / 32][kWarpStage];
     // entry (z = 0, number of harmonics inside the row) and entry (window, |z| = c .. 1): its end in tiles,
     // first and last fundamental, |z| << 14 | fundamentals per thread << 6 | harmonics; entry of a run of
-    // rows: its end in tiles, tiles per row, largest |z|, fundamentals per thread << 6 | harmonics
+    // rows: its end in tiles, tiles per row (or group of rows), largest |z|, rows per tile << 14 (0: one) |
+    // fundamentals per thread << 6 | harmonics
     extern __shared__ int4 ent[];
+    constexpr bool RUNS = MODE != kWindows, TALL = MODE == kTallRuns;
     __shared__ int part[kHsThreads / 32];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int rmax = lim.r_lim[1], most = min(H, rmax);   // harmonics inside a row of the plane
@@ -304,9 +315,17 @@ __global__ void __launch_bounds__(kHsThreads, 2) harmonic_kernel_slope(const flo
             }
             const int e = i - zeros;
             if constexpr (RUNS) {   // rows c / (e + 2) < |z| <= c / (e + 1); the last run: all that are left
-                const int kz = e + 1, hi = c / kz, tile = kHsThreads * hs_q(kz), per_row = (rmax + tile - 1) / tile;
-                sum += 2 * (hi - (kz == runs ? 0 : c / (kz + 1))) * per_row;
-                ent[i] = make_int4(sum, per_row, hi, (hs_q(kz) << 6) | kz);
+                const int kz = e + 1, hi = c / kz, rows = hi - (kz == runs ? 0 : c / (kz + 1));
+                const int tile = kHsThreads * hs_q(kz), per_row = (rmax + tile - 1) / tile;
+                const int cols = (rmax + kHsThreads - 1) / kHsThreads, tall = 2 * ((rows + hs_q(kz) - 1) / hs_q(kz)) * cols;
+                const int blocks = gridDim.x, waves = (2 * rows * per_row + blocks - 1) / blocks;
+                if (TALL && kz <= kHsTall && 2 * ((tall + blocks - 1) / blocks) <= waves) {
+                    sum += tall;
+                    ent[i] = make_int4(sum, cols, hi, (hs_q(kz) << 14) | (1 << 6) | (kHsCases + kz));
+                } else {
+                    sum += 2 * rows * per_row;
+                    ent[i] = make_int4(sum, per_row, hi, (hs_q(kz) << 6) | kz);
+                }
                 continue;
             }
             const int w = e / c, a = c - (e - w * c);
@@ -345,7 +364,7 @@ __global__ void __launch_bounds__(kHsThreads, 2) harmonic_kernel_slope(const flo
             while (passed == 32);
             begin = ent[e - 1].x, en = ent[e];
         }
-        const int kz = en.w & 63, a = en.w >> 14, local = tile - begin;
+        const int body = en.w & 63, a = en.w >> 14, local = tile - begin;
         int z = 0, last = rmax, at = local;   // tile of the row
         if (!RUNS || e < zeros) {
             const int half = (en.x - begin) >> 1;
@@ -355,9 +374,11 @@ __global__ void __launch_bounds__(kHsThreads, 2) harmonic_kernel_slope(const flo
                 at = local < half ? local : local - half;
             }
         } else {
-            const int half = (en.x - begin) >> 1, u = local < half ? local : local - half, row = u / en.y;
-            z = local < half ? en.z - row : row - en.z;
-            at = u - row * en.y;
+            const int half = (en.x - begin) >> 1, u = local < half ? local : local - half, group = u / en.y;
+            const int az = en.z - (TALL ? group * max(a, 1) : group);
+            z = local < half ? az : -az;
+            at = u - group * en.y;
+            if (TALL && a) last = az - (e + 1 < entries ? ent[e + 1].z : 0);   // rows of the run from here on
         }
         const int first = (!RUNS || e < zeros ? en.y : 1) + at * kHsThreads * ((en.w >> 6) & 255);
 #define FDAS_HS_CASE(K)                                                                                                   \
@@ -365,15 +386,22 @@ __global__ void __launch_bounds__(kHsThreads, 2) harmonic_kernel_slope(const flo
         if constexpr (K <= H)                                                                                              \
             hs_tile<K>(P, c, n, bin0, z, first, last, thr, lim, stage[warp], staged, out, max_cand, count);                \
         break;
-        switch (kz) {
+#define FDAS_HS_TALL(K)                                                                                                   \
+    case kHsCases + K:                                                                                                     \
+        if constexpr (TALL && K <= H)                                                                                      \
+            hs_tile<K, hs_q(K), true>(P, c, n, bin0, z, first, last, thr, lim, stage[warp], staged, out, max_cand, count); \
+        break;
+        switch (body) {
             FDAS_HS_CASE(1) FDAS_HS_CASE(2) FDAS_HS_CASE(3) FDAS_HS_CASE(4) FDAS_HS_CASE(5) FDAS_HS_CASE(6) FDAS_HS_CASE(7)
             FDAS_HS_CASE(8) FDAS_HS_CASE(9) FDAS_HS_CASE(10) FDAS_HS_CASE(11) FDAS_HS_CASE(12) FDAS_HS_CASE(13)
             FDAS_HS_CASE(14) FDAS_HS_CASE(15) FDAS_HS_CASE(16) FDAS_HS_CASE(17) FDAS_HS_CASE(18) FDAS_HS_CASE(19)
             FDAS_HS_CASE(20) FDAS_HS_CASE(21) FDAS_HS_CASE(22) FDAS_HS_CASE(23) FDAS_HS_CASE(24) FDAS_HS_CASE(25)
             FDAS_HS_CASE(26) FDAS_HS_CASE(27) FDAS_HS_CASE(28) FDAS_HS_CASE(29) FDAS_HS_CASE(30) FDAS_HS_CASE(31)
             FDAS_HS_CASE(32)
+            FDAS_HS_TALL(1) FDAS_HS_TALL(2)
         }
 #undef FDAS_HS_CASE
+#undef FDAS_HS_TALL
     }
     if (staged) warp_flush(stage[warp], staged, lane, out, max_cand, count);
 }
@@ -414,7 +442,8 @@ cudaError_t launch_hs(int H, const float *P, int m, int64_t n, int64_t bin0, con
             const auto large = harmonic_kernel_rows<hs_q(1)>, small = harmonic_kernel_rows<8>;
             const int64_t tile = (int64_t)kHsThreads * hs_q(1), per_row = (rmax + tile - 1) / tile;
             if ((e = resident_grid((const void *)large, (int64_t)m * per_row, 0, known[0], &grid)) != cudaSuccess) return e;
-            if ((int64_t)m * per_row > 2 * (int64_t)grid) {
+            // (and not for rows that fill less than half of them: 65537 x 4096 218 us, 289 with them)
+            if ((int64_t)m * per_row > 2 * (int64_t)grid && 2 * rmax >= per_row * tile) {
                 large<<<grid, kHsThreads, 0, s>>>(P, c, (int)n, (int)bin0, (int)per_row, thr, lim, out, max_cand, count);
             } else {
                 const int64_t per_row8 = (rmax + kHsThreads * 8 - 1) / (kHsThreads * 8);
@@ -443,21 +472,26 @@ cudaError_t launch_hs(int H, const float *P, int m, int64_t n, int64_t bin0, con
         const size_t table = sizeof(int4) * (32 + (win.count ? (size_t)win.count * c : 32));
         using Kernel = void (*)(const float *, int, int, int, HsThresholds, HsLimits, HsWindows, fdas_harmonic_candidate *,
                                 int64_t, unsigned long long *);
-        auto kernel = [&](auto runs) -> Kernel {
+        auto kernel = [&](auto mode) -> Kernel {
             switch (H) {
-            case 2: return harmonic_kernel_slope<2, runs()>;
-            case 4: return harmonic_kernel_slope<4, runs()>;
-            case 8: return harmonic_kernel_slope<8, runs()>;
-            case 16: return harmonic_kernel_slope<16, runs()>;
-            default: return harmonic_kernel_slope<32, runs()>;
+            case 2: return harmonic_kernel_slope<2, mode()>;
+            case 4: return harmonic_kernel_slope<4, mode()>;
+            case 8: return harmonic_kernel_slope<8, mode()>;
+            case 16: return harmonic_kernel_slope<16, mode()>;
+            default: return harmonic_kernel_slope<32, mode()>;
             }
         };
-        const bool runs = win.count == 0;
-        const Kernel fn = runs ? kernel(std::true_type()) : kernel(std::false_type());
+        // tall tiles where a row fills less than half of its kz = 1 tiles (65537 x 4096 with 2 / 8 / 32
+        // harmonics 278 / 399 / 824 us, without 329 / 468 / 895)
+        const int64_t tile = kHsThreads * hs_q(1), filled = (rmax + tile - 1) / tile * tile;
+        const int mode = win.count ? kWindows : 2 * rmax < filled ? kTallRuns : kRuns;
+        const Kernel fn = mode == kWindows ? kernel(std::integral_constant<int, kWindows>())
+                          : mode == kRuns  ? kernel(std::integral_constant<int, kRuns>())
+                                           : kernel(std::integral_constant<int, kTallRuns>());
         // (the occupancy of the largest table, so that one number serves every call)
-        static std::atomic<int> known[2][6][64];
+        static std::atomic<int> known[3][6][64];
         const int level = 31 - __builtin_clz((unsigned)H);
-        if ((e = resident_grid((const void *)fn, most_tiles, kHsTableBytes, known[runs][level], &grid)) != cudaSuccess) return e;
+        if ((e = resident_grid((const void *)fn, most_tiles, kHsTableBytes, known[mode][level], &grid)) != cudaSuccess) return e;
         fn<<<grid, kHsThreads, table, s>>>(P, c, (int)n, (int)bin0, thr, lim, win, out, max_cand, count);
         return cudaGetLastError();
     }

@@ -56,7 +56,8 @@ def test_crossing_sets(fd, oracle_mod, m, n, bin0, H):
 @pytest.mark.parametrize("m,n,bin0,H", [(4099, 1_025, 0, 32), (4097, 2_000, 3, 8), (20_001, 41, 2, 8),   # rows of |z| > c / H in runs
                                         (8193, 6, 0, 32),             # fewer columns than harmonics
                                         (2_051, 700, 0, 16), (85, 13_000, 210, 2), (3, 3, 0, 2),
-                                        (513, 901, 0, 8), (515, 901, 0, 8), (449, 12_000, 1, 32)])   # long tables over few tiles
+                                        (513, 901, 0, 8), (515, 901, 0, 8), (449, 12_000, 1, 32),     # long tables over few tiles
+                                        (200_001, 20, 0, 2), (60_001, 257, 1, 1), (60_003, 258, 0, 8)])   # short rows, several per tile
 def test_planes_walked_by_rows(fd, oracle_mod, m, n, bin0, H):
     # more rows than the window table takes, and planes beside that limit: every defined sum
     P = synth.noise_plane(m, n, seed=n + H)
