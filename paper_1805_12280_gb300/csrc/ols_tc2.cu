@@ -898,7 +898,7 @@ __global__ void __launch_bounds__(tc2::kThreads, 1)
 {
     Src src = s0;
     src.map = &tmap;
-    tc2_body<CAND, true>(src, a);
+    tc2_body<CAND, !CAND>(src, a);
 }
 
 // Many arrays, one persistent launch: the same items and arithmetic per array as the
@@ -1042,7 +1042,9 @@ cudaError_t launch_ols_tc2(const CUtensorMap *tmap, const OlsArgs &o, const unsi
     // Programmatic dependent launch, as for the FP32 kernel: a block starts on its SM as soon as
     // the block of the launch before has left it, loads the DFT matrices and twiddles, and waits
     // for the end of that launch before it reads the input or writes the output.  us per call, back to
-    // back, before and after: 16384 points 12.3 / 9.4, 65536 17.1 / 14.8, 301000 42.2 / 39.1.
+    // back, before and after: 16384 points 12.3 / 9.4, 65536 17.1 / 14.8, 301000 42.2 / 39.1.  Not with a
+    // threshold: the caller clears the counter just before, so that there is no launch to overlap, and
+    // the attribute with its waits costs 1 % (2^22 points, T_g: 391.2 us with, 387.3 without).
     auto launch = [&](auto kern, int blocks, const auto &src) {
         cudaLaunchAttribute attr{};
         attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -1053,7 +1055,7 @@ cudaError_t launch_ols_tc2(const CUtensorMap *tmap, const OlsArgs &o, const unsi
         cfg.dynamicSmemBytes = tc2::Smem::total;
         cfg.stream = s;
         cfg.attrs = &attr;
-        cfg.numAttrs = 1;
+        cfg.numAttrs = a.cand ? 0 : 1;
         return cudaLaunchKernelEx(&cfg, kern, *tmap, a, src);
     };
     const int n_sp = (nseg + 1) / 2;
