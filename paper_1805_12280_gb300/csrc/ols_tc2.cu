@@ -435,10 +435,7 @@ __device__ __forceinline__ void tc2_body(const Src &src, const tc2::Args &a)
     __syncthreads();
     tmem_fence_after_sync();
     const uint32_t tmem = *tslot;
-    if constexpr (PDL) {
-        launch_dependents();    // this block holds its tensor memory (see launch_ols_tc2)
-        wait_prerequisites();   // before any output is written
-    }
+    if constexpr (PDL) wait_prerequisites();   // before any output is written
 
     if (warp < 4) {
         // ---------------- product group: forward FFTs, X . H_z into the stage-1 operand ----------------
@@ -875,6 +872,7 @@ __device__ __forceinline__ void tc2_body(const Src &src, const tc2::Args &a)
                 }
             }
         }
+        if constexpr (PDL) launch_dependents();   // the last tiles remain (see launch_ols_tc2)
         // nothing may be in flight when the block leaves: the copies issued land first
         if (seg_issued) mbar_wait_bounded(&bar[B_SEG_FULL], (seg_issued - 1) & 1, kWaitLimitNs);
         for (uint32_t i = (tH > NH ? tH - NH : 0); i < tH; ++i)
@@ -1043,7 +1041,11 @@ cudaError_t launch_ols_tc2(const CUtensorMap *tmap, const OlsArgs &o, const unsi
     // Programmatic dependent launch, as for the FP32 kernel: a block starts on its SM as soon as
     // the block of the launch before has left it, loads the DFT matrices and twiddles, and waits
     // for the end of that launch before it reads the input or writes the output.  us per call, back to
-    // back, before and after: 16384 points 12.3 / 9.4, 65536 17.1 / 14.8, 301000 42.2 / 39.1.  Not with a
+    // back, before and after: 16384 points 12.3 / 9.5, 65536 17.9 / 14.8, 301000 43.0 / 38.7.  A waiting block
+    // keeps its SM from other streams, so a block lets the next launch start only when its last template
+    // is on the way (one of 2^22 points beside sixteen FP32 calls of 2^14 on a second stream: 604 us without
+    // the overlap, 579 when blocks let go at their start, 567 so; beside one FP32 call of 301000 points
+    // both 301000: 96.8 / 99.5 / 99.3; four streams of 16384 points: 29.7 / 30.6 / 30.6).  Not with a
     // threshold: the caller clears the counter just before, so that there is no launch to overlap, and
     // the attribute with its waits costs 1 % (2^22 points, T_g: 391.2 us with, 387.3 without).
     auto launch = [&](auto kern, int blocks, const auto &src) {
