@@ -389,11 +389,13 @@ def run_fdas(args):
     roofline_alu["sms"] = sms
     roofline_alu["frac"] = roofline_alu["achieved"] / roofline_alu["peak"]
     if rank == 0:
+        share_blocks = fd.fdas_plan_share_blocks(plan.handle, n)   # 0: a block per segment and template group
         line = {"metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": args.steps,
                 "warmup": args.warmup, "ms_per_step": ms_per_step, "higher_is_better": True, "scaling": "weak",
                 "vs_baseline": value / PAPER_ARRAYS_PER_S, "dtype": "f32", "data": "synthetic",
                 "config": workload_config(args, n, h.shape[1]),
-                "tpl_per_cta_used": fd.fdas_plan_tpl_per_cta(plan.handle, n),
+                "tpl_per_cta_used": None if share_blocks else fd.fdas_plan_tpl_per_cta(plan.handle, n),
+                "share_blocks_used": share_blocks,
                 "plane_gbs": 4.0 * m * n * world / (ms_per_step / 1e3) / 1e9,
                 "model_tflops": model_flops(n, m, args.seg_len, h.shape[1]) * world / (ms_per_step / 1e3) / 1e12,
                 "roofline": roofline, "roofline_alu": roofline_alu, "cpu_baseline": cpu, "e2e": e2e,

@@ -119,11 +119,19 @@ int fdas_plan_describe(fdas_plan p, fdas_plan_desc *desc);
 
 /* Templates per thread block that fdas_convolve uses for an array of n points (the plan's
  * fixed G, or the per-call choice when the plan was created with tpl_per_cta = 0; a grouped
- * plan applies the same rule to each template group and its segment count; where the blocks of
- * a plane's launch take equal shares of its work instead, this is what the rule would have been).
+ * plan applies the same rule to each template group and its segment count).  Where
+ * fdas_plan_share_blocks is not 0, the call's blocks do not take groups of templates, and this
+ * is the group that the threshold form of the call takes.
  * Returns G >= 1, or a negative error code (INVALID_ARG for a null plan or n outside
  * [1, n_max]).  Host only; no CUDA call. */
 int fdas_plan_tpl_per_cta(fdas_plan p, int64_t n);
+
+/* Blocks among which fdas_convolve divides the (segment, template) units of an array of n
+ * points equally, in one launch, or 0 where each block takes one segment's template group
+ * (fdas_plan_tpl_per_cta).  Equal shares are chosen per call, by FP32 plans created with
+ * tpl_per_cta = 0; a grouped plan chooses for each template group, and this is not 0 if any of
+ * its launches takes shares.  Errors and host-only as above. */
+int fdas_plan_share_blocks(fdas_plan p, int64_t n);
 
 /*
  * fdas_convolve -- power plane of one array (the hot path).

@@ -236,6 +236,13 @@ int launch_range(fdas_plan p, const CUtensorMap *map, fdas::OlsArgs a, int64_t s
     return FDAS_OK;
 }
 
+// Segments of a template group's launch; one writes the zero prefix of an array that ends in it.
+int64_t group_segments(const fdas_plan_s::Group &gr, int64_t n)
+{
+    const int64_t span = n - gr.min_shift;
+    return span > 0 ? (span + gr.S - 1) / gr.S : 1;
+}
+
 // All segments of every template group: one launch per group.
 int launch_all(fdas_plan p, const CUtensorMap *map, const fdas::OlsArgs &a0, int64_t n, cudaStream_t stream)
 {
@@ -249,8 +256,7 @@ int launch_all(fdas_plan p, const CUtensorMap *map, const fdas::OlsArgs &a0, int
         a.K = gr.K;
         a.rows = p->d_rows + gr.first;
         a.shifts = p->d_shifts + gr.first;
-        const int64_t span = n - gr.min_shift;
-        const int64_t nseg = span > 0 ? (span + gr.S - 1) / gr.S : 1;   // one segment writes the zero prefix
+        const int64_t nseg = group_segments(gr, n);
         a.G = call_G(p, nseg, gr.count);
         a.blocks = call_blocks(p, nseg, gr.count, a.cand != nullptr);
         cudaError_t e = fdas::launch_ols_fp32(p->L, map, a, (int)nseg, stream);
@@ -897,6 +903,17 @@ int fdas_plan_tpl_per_cta(fdas_plan p, int64_t n)
     if (!p) return fail(FDAS_ERR_INVALID_ARG, "null plan");
     if (n < 1 || n > p->n_max) return fail(FDAS_ERR_INVALID_ARG, "n=%lld outside [1, n_max=%lld]", (long long)n, (long long)p->n_max);
     return call_G(p, n_segments(p, n), p->M);
+}
+
+int fdas_plan_share_blocks(fdas_plan p, int64_t n)
+{
+    if (!p) return fail(FDAS_ERR_INVALID_ARG, "null plan");
+    if (n < 1 || n > p->n_max) return fail(FDAS_ERR_INVALID_ARG, "n=%lld outside [1, n_max=%lld]", (long long)n, (long long)p->n_max);
+    if (p->ngroups <= 1 && !p->d_rows) return call_blocks(p, n_segments(p, n), p->M, false);
+    int blocks = 0;
+    for (int g = 0; g < p->ngroups && !blocks; ++g)
+        blocks = call_blocks(p, group_segments(p->groups[g], n), p->groups[g].count, false);
+    return blocks;
 }
 
 int fdas_convolve_batch(fdas_plan p, int count, const void *const *ins, const int64_t *ns, float *const *outs,

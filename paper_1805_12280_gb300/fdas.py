@@ -89,6 +89,7 @@ SIGNATURES = {
     "fdas_plan_create": (_I, [ctypes.POINTER(_P), _I64, _P, _I, _I, ctypes.POINTER(fdas_opts)]),
     "fdas_plan_describe": (_I, [_P, ctypes.POINTER(fdas_plan_desc)]),
     "fdas_plan_tpl_per_cta": (_I, [_P, _I64]),
+    "fdas_plan_share_blocks": (_I, [_P, _I64]),
     "fdas_convolve": (_I, [_P, _P, _I64, _P, _P]),
     "fdas_convolve_host": (_I, [_P, _P, _I64, _P, _P]),
     "fdas_convolve_batch": (_I, [_P, _I, ctypes.POINTER(_P), ctypes.POINTER(_I64), ctypes.POINTER(_P), _P]),
@@ -168,6 +169,12 @@ def fdas_plan_tpl_per_cta(plan: int, n: int) -> int:
     g = load().fdas_plan_tpl_per_cta(_P(plan), int(n))
     _check(min(g, 0), "fdas_plan_tpl_per_cta")
     return g
+
+
+def fdas_plan_share_blocks(plan: int, n: int) -> int:
+    b = load().fdas_plan_share_blocks(_P(plan), int(n))
+    _check(min(b, 0), "fdas_plan_share_blocks")
+    return b
 
 
 def fdas_selftest_wait_timeout(plan: int, limit_ms: float, stream: int = 0) -> None:

@@ -39,3 +39,25 @@ def test_equal_shares_match_groups(L, m, k, group):
             auto.status()
             fixed.status()
             assert torch.equal(a, b)
+
+
+def test_the_split_a_call_takes_is_reported():
+    # the resident blocks where a call takes equal shares, at both ends of their range; 0: template groups
+    import paper_1805_12280_gb300 as fd
+    fd.load()
+    h = _bank(85, 421, 1)
+    with fd.Plan(h, n_max=1 << 22) as plan, fd.Plan(h, n_max=1 << 22, tpl_per_cta=17) as fixed, \
+            fd.Plan(h, n_max=1 << 22, precision=fd.FDAS_PREC_TC_DFT2) as tc:
+        slots, S = plan.desc.batch_blocks, plan.desc.seg_step
+        first = -(-7 * slots // 85)
+        for nseg, shares in ((1, 0), (first - 1, 0), (first, slots), (45 * slots // 85, slots), (45 * slots // 85 + 1, 0)):
+            assert fd.fdas_plan_share_blocks(plan.handle, nseg * S) == shares
+            assert fd.fdas_plan_tpl_per_cta(plan.handle, nseg * S) >= 1
+            for other in (fixed, tc):
+                assert fd.fdas_plan_share_blocks(other.handle, nseg * S) == 0
+        for bad in (0, (1 << 22) + 1):
+            with pytest.raises(fd.FdasError) as e:
+                fd.fdas_plan_share_blocks(plan.handle, bad)
+            assert e.value.code == fd.fdas.FDAS_ERR_INVALID_ARG
+    with fd.Plan(h, n_max=1 << 22, group_support=1) as plan:
+        assert fd.fdas_plan_share_blocks(plan.handle, 1) == 0
