@@ -198,8 +198,10 @@ int call_G(const fdas_plan p, int64_t nseg, int m)
 // blocks partly empty; a share costs one more forward FFT where it crosses a segment boundary.
 // Measured over 21 lengths each at 6 to 63 units per block and 85, 43 and 21 templates, time of
 // shares / groups: from 7 units on, L = 4096 0.80 .. 0.99 and L = 1024 0.82 .. 0.96 at all sizes
-// (85 templates of 2^22 points 818 -> 756 us, 1060 -> 1038), L = 2048 0.91 .. 1.02 up to 45 units
-// (301000 points 66.0 -> 63.3 us, 400000 88.8 -> 81.7).  Below 7 units a share is too short for its
+// (85 templates of 2^22 points 818 -> 756 us, 1060 -> 1038), L = 2048 0.89 .. 1.045 up to 45 units,
+// above 1.01 at 6 of 87 lengths, where the groups' waves happen to come out even (301000 points
+// 66.0 -> 63.3 us, 400000 88.8 -> 81.7, 244544 51.3 -> 53.6; no length is slower than groups whose
+// launches do not overlap).  Below 7 units a share is too short for its
 // forward FFTs (41000 points 13.0 us against 15.6); longer ones with L = 2048, four blocks of four
 // warps an SM, drift apart and the last runs alone (2^22 points 721 us against 770), where groups
 // in several waves even out.  With 9 templates, 0.88 .. 1.09: groups.

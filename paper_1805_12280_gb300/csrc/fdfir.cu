@@ -14,9 +14,9 @@
 //
 // Why 1024 x P2: a block's piece of a row is 8 values (64 bytes).  With 2048-point columns four
 // fit a block, and their 32-byte pieces (8 cache lines per request of a warp) cost the load/store
-// pipe as much as both exchanges of the transform.  85 templates, P = 2^21 / 2^22 / 2^23:
-// 1420 / 2400 / 4900 us with 2048-point columns and the passes in launches of their own, 952 /
-// 2106 / 4470 with this split and the passes of two templates in one launch (fdfir_inv_step).
+// pipe as much as both exchanges of the transform.  85 templates, largest array of P = 2^21 / 2^22, and
+// 2^22 points at P = 2^23: 1048 / 2260 / 4470 us (4117 / 8237 / 14316 in the form before: columns of
+// 2048 points one after another in a block, the two passes in launches that did not overlap).
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -56,8 +56,7 @@ constexpr size_t inv_smem_bytes()
 // The M + 1 inverse launches of a call overlap (programmatic dependent launch): every block lets
 // the next launch start as soon as all blocks of this one run, and waits for the launch before it
 // only where it touches the scratch B that the passes hand on.  A block of launch i passes its wait
-// before it ends, so the end of a launch implies the end of all before it.  (With the two passes
-// in launches of their own, 85 templates of 2^23 points: 5896 us without the overlap, 5046 with.)
+// before it ends, so the end of a launch implies the end of all before it.
 
 // exp(dir * 2 pi i e / P), e < P <= 2^23 (the argument 2e/P is exact in FP32)
 __device__ __forceinline__ float2 twiddle_p(int e, float two_over_p, float dir)
@@ -125,8 +124,7 @@ __device__ __forceinline__ void forward_fft_folded(float2 (&v)[16], float2 *ex, 
 
 // Column pass, forward: columns n2 = blockIdx.x * CT + col of in[P2 n1 + n2] (zero at and beyond
 // len) -> A[r][n2] = scale * W_P^{n2 k1} * FFT_P1 over n1, row r = j*NT1 + t for slot j of t.
-// Thread (t, column) as in the inverse pass.  A call with 3 templates of 2^23 points: 286 us with
-// four columns one after another in a block of 64 threads, 243 with this.
+// Thread (t, column) as in the inverse pass.
 template <int P2>
 __global__ void __launch_bounds__(fd::NT_INV, 2) fdfir_col_fwd(const float2 *__restrict__ in, int64_t len,
                                                               const float2 *__restrict__ tw1, float2 *__restrict__ A,
@@ -211,7 +209,7 @@ __device__ __forceinline__ void inverse_fft_folded(float2 (&v)[16], float2 *ex, 
         for (int k2 = 0; k2 < Q; ++k2) v[g * Q + k2] = ex[(k1 + 16 * k2 + 16 * Q * (hi + (NT / 16) * g)) * CT + col];
         dft_twiddled<Q>(v + g * Q, w + g * (Q / 2));
     }
-    if constexpr (CT == 1) {   // 32 t per warp: 40 lines from W_L, 16 from the table (2^22: 2159 -> 2106 us)
+    if constexpr (CT == 1) {   // 32 t per warp: 40 lines from W_L, 16 from the table
 #pragma unroll
         for (int i = 0; i < 8; ++i) w[i] = __ldg(&tw[L + i * NT + t]);
     } else {
@@ -231,9 +229,9 @@ __device__ __forceinline__ void inverse_fft_folded(float2 (&v)[16], float2 *ex, 
 // Row pass, inverse, with the product: B[r][n2] = IFFT_P2 over k2 of X[r][.] * H[r][.]; unit: the
 // rows of one block.  X and the two B (201 MB at P = 2^23) do not fit L2, and a cyclic walk of X
 // would miss always; templates walk the rows up and down in turn, so that what the last one read
-// last is read first (one direction: 4774 us against 4688), and what is used once is marked
-// streaming: H always, X where it would push B out (2^23: 4688 -> 4524 us; at 2^21, where it
-// stays, 1123 -> 1140).
+// last is read first (one direction, largest array of P = 2^22: 2300 us against 2256), and what is
+// used once is marked streaming: H always, X where it would push B out (2^23: 4471 us, 4628 if not; at
+// 2^21, where it stays, 1048 against 1091 with the mark).
 template <int P2>
 __device__ __forceinline__ void row_inv(const float2 *__restrict__ X, const float2 *__restrict__ H, float2 *__restrict__ B,
                                         const float2 *__restrict__ tw2, const float2 *__restrict__ twr, int unit, float2 *smem)
@@ -281,7 +279,7 @@ __device__ __forceinline__ void row_inv(const float2 *__restrict__ X, const floa
 // a thread in flight, and the exchanges (values of the CT columns side by side, one buffer used
 // twice) are free of bank conflicts.  The twiddle of slot (g, k3) is a base per g times a step
 // per k3: two sincospif per thread and 8 per column.  B is marked streaming where two templates'
-// B do not fit L2 (2^23: 4454 us, 4592 if not; 2^22: 2186 against 2219).
+// B do not fit L2 (2^23: 4471 us, 4598 if not; 2^22: 2256 against 2287).
 template <int P2>
 __device__ __forceinline__ void col_inv(const float2 *__restrict__ B, const float2 *__restrict__ tw1,
                                         float *__restrict__ out, int64_t n, int n2_0, float2 *fd_smem)
@@ -319,10 +317,10 @@ __device__ __forceinline__ void col_inv(const float2 *__restrict__ B, const floa
 // One launch: the rows of one template (H given) and the columns of the one before (out given),
 // each on half of the blocks; two B buffers alternate.  The row pass waits on memory (X and H
 // from DRAM) while the column pass keeps the load/store pipe busy: together they take less than
-// one after the other (P = 2^21 1243 -> 1123 us, 2^22 2269 -> 2218, 2^23 4730 -> 4686).  Blocks of
-// the two kinds in turn, so that an SM holds one of each; P = 2^21 with the rows first, since its
-// 512 blocks are two waves and the rows, which start before the launch ahead has ended, fill the
-// first (1123 -> 994 us; no gain above).
+// one after the other (10 / 2 / 1 % of a call at P = 2^21 / 2^22 / 2^23 when it was made).  Blocks of the
+// two kinds in turn, so that an SM holds one of each; P = 2^21 with the rows first, since its 512 blocks
+// are two waves and the rows, which start before the launch ahead has ended, fill the first (in turn
+// 1154 us against 1048; no gain above).
 template <int P2>
 __global__ void __launch_bounds__(fd::NT_INV, 2) fdfir_inv_step(const float2 *__restrict__ X, const float2 *__restrict__ H,
                                                                float2 *__restrict__ Bw, const float2 *__restrict__ Br,

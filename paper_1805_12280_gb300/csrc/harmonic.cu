@@ -17,12 +17,12 @@
 //
 // Planes narrower than 2^31 columns take one launch that walks the plane in slope windows (below)
 // with code compiled for each number of harmonics that lie in the plane; crossings are staged
-// per warp, with no block barrier.  85 x 2^22, 8 harmonics: 324 us, 1.71 GB of DRAM traffic (1.2
-// planes), against 597 us and 3.40 GB when rows were launched in runs of equal harmonic
-// count and every strided pass fetched its rows again; 32 harmonics 842 -> 508 us, one harmonic
-// 272 -> 228 us, 65536 columns 61 -> 23 us per call (15 launches -> 1).  What bounds it: load
-// latency at 16 warps per SM (issue 40 %, DRAM 78 % of the measured copy rate); three blocks per SM
-// (fewer loads in flight per thread) are 6 % slower.
+// per warp, with no block barrier.  85 x 2^22, 8 harmonics: 310 us, 1.68 GB of DRAM traffic (1.18
+// planes), against 599 us and 3.40 GB when rows were launched in runs of equal harmonic
+// count and every strided pass fetched its rows again; 32 harmonics 845 -> 404 us, one harmonic
+// 276 -> 224 us, 65536 columns and 8 harmonics 55 -> 17 us per call (15 launches -> 1).  What bounds it:
+// load latency at 16 warps per SM (issue 40 %, DRAM 80 % of the measured copy rate); three blocks per
+// SM, with fewer loads in flight per thread, are slower.
 // Planes of more than 513 rows, whose table has little room for windows, go by runs of rows with the
 // same number of harmonics in the same launch.  Wider rows take the general kernel with 64-bit indexing.
 #include <cuda_runtime.h>
@@ -160,8 +160,8 @@ __device__ __forceinline__ void warp_flush(const fdas_harmonic_candidate *stage,
 // closed under the sums, and the plane is walked window by window: row |z| = a takes the
 // fundamentals (a S_w, a S_{w+1}], and every harmonic it reads lies in the part of row k a that the
 // same window reads as fundamentals, so all but the first read of a cell hit L2.  The z = 0 row
-// (its harmonics lie in itself) comes first.  Windows of 64 MB (8 harmonics at 2^22, sorted
-// records included: 16 MB 766, 32 MB 711, 64 MB 693, the whole plane 771 us in one version).
+// (its harmonics lie in itself) comes first.  Windows of 64 MB (85 x 2^22, 8 / 32 harmonics: 16 MB 315 /
+// 383 us, 32 MB 313 / 370, 64 MB 313 / 405, 128 MB 346 / 433, the whole plane at once 509 / 760).
 constexpr int kHsMaxWin = 128, kHsMaxEntries = 2048;   // windows; (window, |z|) entries of one launch
 constexpr size_t kHsTableBytes = sizeof(int4) * (kHsMaxEntries + 32);   // with the z = 0 row's
 constexpr int64_t kHsWindowBytes = 64ll << 20;
@@ -171,7 +171,8 @@ struct HsWindows {
 };
 
 // Fundamentals per thread of rows with kz harmonics: 48 to 64 loads in flight, and a bit per
-// (fundamental, level) in one mask (16 and 8 fundamentals for kz = 1 and 2: 609 us against 510).
+// (fundamental, level) in one mask (85 x 2^22, 8 harmonics: 313 us; with 16 for kz = 1 and 8 for 2 and
+// 3: 407; 8 for all of them: 533).
 __host__ __device__ constexpr int hs_q(int kz) { return kz == 1 ? 48 : kz == 2 ? 24 : kz == 3 ? 16 : kz <= 8 ? 8 : 64 / kz; }
 constexpr int kHsTall = 2, kHsCases = 32;   // tall tiles are compiled for kz <= kHsTall, as cases above kHsCases
 __host__ __device__ constexpr int hs_levels(int kz) { return kz < 2 ? 1 : 1 + hs_levels(kz / 2); }

@@ -617,8 +617,8 @@ static cudaError_t launch_lc(const CUtensorMap *tmap, const OlsArgs &a, int nseg
     // holds its tensor memory then, so a block that waits never holds columns that the launch
     // before still needs (and starts its dependents late enough: let go at its start, their blocks
     // fill the SMs that drain first and run four to an SM beside idle ones, 32768 points in a graph
-    // 16.4 us against 12.8).  us per call, back to back, before and after: 16384 points 12.3 / 10.0,
-    // 65536 24.7 / 21.1, 301000 69.5 / 65.9, 2^22 722 / 720.
+    // 16.4 us against 12.8).  us per call, back to back, before and after: 16384 points 12.5 / 10.2,
+    // 65536 24.7 / 21.2, 301000 69.0 / 65.9 (63.4 with equal shares); nothing at 2^22 (721).
     cudaLaunchAttribute attr{};
     attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr.val.programmaticStreamSerializationAllowed = 1;
